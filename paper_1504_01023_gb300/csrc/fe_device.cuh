@@ -8,6 +8,7 @@
 
 #include "fe_dword.cuh"
 #include "fe_f64int.cuh"
+#include "fe_fixed.cuh"
 #include "fe_internal.h"
 
 namespace fe {

@@ -1,15 +1,15 @@
 // Explicit kernel tables: every (kind, coefficient mode, input layout, output
 // layout) combination of one element type, precision and rule.
 #pragma once
-#include "fe_kernels.cuh"
+#include "fe_stream.cuh"
 
 #define FE_ELEM_CASE(ET, PREC, QUAD, KD, CP, IL, OL)                                  \
     if (kind == KD && cpq == CP && inl == IL && outl == OL)                          \
         return reinterpret_cast<const void *>(&fe::elem_kernel<ET, KD, PREC, QUAD, CP, IL, OL>);
-// FP64 tetrahedra: the register-capped variant of the main kernel.
+// FP64 tetrahedra: the warp-at-a-time kernel or the register-capped tile kernel
+// (f64_tet_kernel).
 #define FE_F64T_CASE(ET, PREC, QUAD, KD, CP, IL, OL)                                  \
-    if (kind == KD && cpq == CP && inl == IL && outl == OL)                          \
-        return reinterpret_cast<const void *>(&fe::elem_kernel_f64t<KD, QUAD, CP, IL, OL>);
+    if (kind == KD && cpq == CP && inl == IL && outl == OL) return fe::f64_tet_kernel<KD, QUAD, CP, IL, OL>();
 // Double-word tetrahedra: the register-capped variant of the main kernel for
 // per-element coefficients (dw_tet_kernel).
 #define FE_DWT_CASE(ET, PREC, QUAD, KD, CP, IL, OL)                                   \

@@ -48,15 +48,13 @@ template <class XS> __device__ __forceinline__ V3<DW> dw_edge_vec(const XS &x, i
 // ---------------------------------------------------------------------------
 template <int ET, int KIND, int PREC, int QUAD, int CPQ> struct ElemMath;
 
-// Tetrahedron, FP64 (Algorithm 3 in double). The Laplace kind and the generic
-// kind with per-element coefficients run the scalings of the coefficients and of
-// det J and the products of the cofactors (TetF64's OM and OX groups) in integer
-// instructions that report special cases (the same IEEE results): they relieve
-// the double pipe (6M generic tetrahedra 3.94 -> 4.04 Gelem/s with the cofactor
-// products, Laplace 9.26 -> 9.65). Integer edges or row sums lengthen the chain
-// of dependent additions and measured slower even in the reporting form (generic:
-// sums 0.83x, edges and sums 0.76x; Laplace 0.84x, 0.71x). Per-point
-// coefficients take the general products.
+// Tetrahedron, FP64 (Algorithm 3 at double accuracy). The Laplace kind and the
+// generic kind with per-element coefficients run in block fixed point (TetFx):
+// the double pipe, which bounded both at 0.83-0.90 of its rate (136 and 49 double
+// instructions per element, 6M elements 4.17 and 10.65 Gelem/s), keeps the edge
+// differences, one reciprocal and one conversion per distinct result (34 and 26).
+// Elements outside its windows, and generic per-point coefficients, take the
+// double pipe throughout.
 template <int KIND, int QUAD, int CPQ> struct ElemMath<TET, KIND, FP64, QUAD, CPQ> {
     template <class XS, class CS>
     __device__ __forceinline__ static uint8_t run(const XS &x, const CS &c, double A[16], double b[4], bool &poor) {
@@ -78,30 +76,48 @@ template <int KIND, int QUAD, int CPQ> struct ElemMath<TET, KIND, FP64, QUAD, CP
             tet_generic_products<double, QUAD, CPQ>(g, V, c, A, b);
             return is_neg(geo.det) ? 2 : 0;
         } else {
-            // scalings in integer instructions; an element that meets a special
-            // operand or product there is redone on the double pipe (one branch
-            // per element, never taken on ordinary data)
-            using TF = TetF64<F64<false>, F64<true>, F64<true>, F64<false>>;
-            using TH = TetF64<F64<false>, F64<false>, F64<false>, F64<false>>;
-            double a[3][3], det;
-            bool sp = false;
-            if (!TF::geometry(x, a, det, sp)) return zero(A, b);
-            if constexpr (KIND == POISSON)
-                TF::template poisson<QUAD, CPQ>(a, det, c, A, b, sp);
-            else
-                TF::template generic<QUAD>(a, det, c, A, b, sp);
-            if (sp) {
-                // from the inputs again (the compiler barrier keeps the first pass's
-                // values from being held for this path)
-                asm volatile("" ::: "memory");
-                double a2[3][3], det2;
-                TH::geometry(x, a2, det2, sp);
-                if constexpr (KIND == POISSON)
-                    TH::template poisson<QUAD, CPQ>(a2, det2, c, A, b, sp);
-                else
-                    TH::template generic<QUAD>(a2, det2, c, A, b, sp);
+            TetFx fx;
+            if (fx.geometry(x)) {
+                bool ok = true;
+                if constexpr (KIND == POISSON) {
+                    fx.laplace(A);
+                    poisson_b(fx.volume(), c, b);
+                } else {
+                    ok = fx.template generic<QUAD == Q_TET4>(c, A, b);
+                }
+                if (ok) return fx.neg ? 2 : 0;
             }
-            return is_neg(det) ? 2 : 0;
+            // outside the fixed-point windows: the double pipe, from the inputs again
+            // (the compiler barrier keeps the first pass's values from being held)
+            asm volatile("" ::: "memory");
+            return run_double(x, c, A, b);
+        }
+    }
+    // Every operation on the double pipe.
+    template <class XS, class CS>
+    __device__ __forceinline__ static uint8_t run_double(const XS &x, const CS &c, double A[16], double b[4]) {
+        using TH = TetF64<F64<false>, F64<false>, F64<false>, F64<false>>;
+        double a[3][3], det;
+        bool sp = false;
+        if (!TH::geometry(x, a, det, sp)) return zero(A, b);
+        if constexpr (KIND == POISSON)
+            TH::template poisson<QUAD, CPQ>(a, det, c, A, b, sp);
+        else
+            TH::template generic<QUAD>(a, det, c, A, b, sp);
+        return is_neg(det) ? 2 : 0;
+    }
+    // Load vector of the Laplace kind: b_r = V sum_q w_q d0_q phi_r(q). Four points:
+    // phi_r(q) = A + (B - A) [q == r], so b_r = V (w A sum_q d0_q + w (B - A) d0_r).
+    template <class CS> __device__ __forceinline__ static void poisson_b(double V, const CS &c, double b[4]) {
+        if constexpr (!CPQ || Rule<QUAD>::NQ == 1) {
+            const double vd = (V * c(0)) * tet_sums<QUAD>().m[0];   // m_r = W / 4 for both rules
+#pragma unroll
+            for (int r = 0; r < 4; ++r) b[r] = vd;
+        } else {
+            const double d[4] = {c(0), c(1), c(2), c(3)};
+            const double s = ((d[0] + d[1]) + (d[2] + d[3])) * (Rule<QUAD>::w(0) * kTet4A);
+#pragma unroll
+            for (int r = 0; r < 4; ++r) b[r] = fma(d[r], Rule<QUAD>::w(0) * (kTet4B - kTet4A), s) * V;
         }
     }
     __device__ __forceinline__ static uint8_t zero(double A[16], double b[4]) {
@@ -1802,18 +1818,16 @@ __global__ void __launch_bounds__(ET == TET && PREC != DWORD ? 512 : 256,
     elem_tiles<ET, KIND, PREC, QUAD, CPQ, INL, OUTL>(p, &tm, &fn);
 }
 
-// The same kernel for FP64 tetrahedra with fewer registers per thread. Generic
-// kind 104 (6M tetrahedra 4.10 -> 4.18 Gelem/s against 128 registers; 96 and 80
-// spilled more and measured 4.14 and 4.04): still four warps per SM
-// sub-partition, but the allocation under the bound keeps the double pipe busier
-// (ncu 87.3% -> 89.7%). Laplace kind 80 (6M TET1 9.77 -> 10.58 Gelem/s against
-// 100; 88 and 72 measured 10.29 and 10.52): six warps per sub-partition instead
-// of five to cover the chains of the integer-instruction products. ptxas gets
-// both the block bound (.maxntid 512) and the register bound (.maxnreg); with the
-// register bound alone it allocates differently (the generic element-contiguous
-// kernel spilled 360 bytes instead of 20).
+// The same kernel for FP64 tetrahedra with fewer registers per thread: Laplace kind
+// 56 (3M TET1, element-contiguous: 48 registers 14.2, 56 16.5, 64 15.1, 80 13.8
+// Gelem/s), generic kind 96 (3M TET4, fixed point: 64 registers 6.8, 80 8.7, 96
+// 9.2, 104 8.8, 128 8.9), generic per-point coefficients 104 (double pipe; 128, 96
+// and 80 measured slower). ptxas gets both the block bound (.maxntid 512) and the
+// register bound (.maxnreg); with the register bound alone it allocates
+// differently (the generic element-contiguous kernel spilled 360 bytes instead of
+// 20).
 template <int KIND, int QUAD, int CPQ, int INL, int OUTL>
-__global__ void __launch_bounds__(512) __maxnreg__(KIND == POISSON ? 80 : 104)
+__global__ void __launch_bounds__(512) __maxnreg__(KIND == POISSON ? 56 : (CPQ ? 104 : 96))
     elem_kernel_f64t(const ElemParams p, const __grid_constant__ TmaMaps tm, const __grid_constant__ CoefFn fn) {
     elem_tiles<TET, KIND, FP64, QUAD, CPQ, INL, OUTL>(p, &tm, &fn);
 }

@@ -167,10 +167,18 @@ static int na_out(fe_elem_type type, int outl) {
     return out_packed(outl) ? ns * (ns + 1) / 2 : ns * ns;
 }
 
-static int64_t smem_bytes(fe_elem_type type, const fe_elem_args *a, int outl, int B) {
+// The warp-at-a-time kernel of FP64 tetrahedra (fe_stream.cuh, f64_tet_kernel).
+static bool stream_ok(fe_elem_type type, const fe_elem_args *a, int outl) {
+    const int cpq = cpq_of(a);
+    return type == FE_TET && a->prec == FE_FP64 && a->coords_layout == FE_LAYOUT_AOS && outl == AOS &&
+           (cpq == 0 || (cpq == 1 && a->kind == FE_POISSON));
+}
+
+static int64_t smem_bytes(fe_elem_type type, const fe_elem_args *a, int outl, int B, int tpe) {
     // tetrahedra with a node table read straight from global memory (gather_kernel)
     if (a->coords_layout == FE_LAYOUT_INDEXED && type == FE_TET) return 0;
     const int ns = ns_of(type), nc = nc_of(type, a), cs = csize(a->prec);
+    if (tpe == 1 && stream_ok(type, a, outl)) return int64_t(B) * (96 + 8 * nc);   // results leave from registers
     auto r16 = [](int64_t v) { return (v + 15) / 16 * 16; };
     const int64_t geo = a->coords_layout == FE_LAYOUT_INDEXED ? r16(int64_t(B) * ns * 4) : int64_t(B) * 3 * ns * 8;
     const int64_t in = geo + r16(int64_t(B) * nc * cs),
@@ -287,7 +295,7 @@ fe_status launch_set(fe_ctx *ctx, fe_elem_type type, const fe_elem_args *a, cons
     if (!k) return set_error(ctx, FE_ERR_UNSUPPORTED, "no kernel for this combination");
     const int threads = shape_threads(sh.block, sh.tpe);
     if (!threads) return set_error(ctx, FE_ERR_INVALID_ARG, "bad launch shape");
-    const int64_t smem = smem_bytes(type, a, outl, sh.block);
+    const int64_t smem = smem_bytes(type, a, outl, sh.block, sh.tpe);
     if (smem + kStaticSmem > ctx->max_smem_optin)
         return set_error(ctx, FE_ERR_UNSUPPORTED, "shared memory of this launch shape too large");
     {
@@ -967,7 +975,7 @@ fe_status fe_set_launch_shape(fe_ctx *ctx, fe_elem_type type, const fe_elem_args
         return set_error(ctx, FE_ERR_UNSUPPORTED, "several threads per element: 2 for prisms, 4 or 16 for tetrahedra, "
                                                   "6 for prisms, with element-contiguous coordinates and outputs, "
                                                   "coefficient arrays and the QSS order only");
-    if (smem_bytes(type, args, out_mode(out), B) + kStaticSmem > ctx->max_smem_optin)
+    if (smem_bytes(type, args, out_mode(out), B, t) + kStaticSmem > ctx->max_smem_optin)
         return set_error(ctx, FE_ERR_UNSUPPORTED, "shared memory of this launch shape too large");
     ctx->shapes[shape_key(type, args, out)] = Shape{B, shape->persistent, t};
     save_tuning_cache(ctx);
@@ -981,7 +989,7 @@ fe_status fe_set_shape(fe_ctx *ctx, fe_elem_type type, const fe_elem_args *args,
     if (st != FE_OK) return st;
     if (block_threads < 32 || block_threads > max_block(type, args->prec) || block_threads % 32 || (persistent != 0 && persistent != 1))
         return set_error(ctx, FE_ERR_INVALID_ARG, "bad launch shape");
-    if (smem_bytes(type, args, out_mode(out), block_threads) + kStaticSmem > ctx->max_smem_optin)
+    if (smem_bytes(type, args, out_mode(out), block_threads, 1) + kStaticSmem > ctx->max_smem_optin)
         return set_error(ctx, FE_ERR_UNSUPPORTED, "shared memory of this launch shape too large");
     ctx->shapes[shape_key(type, args, out)] = Shape{block_threads, persistent};
     save_tuning_cache(ctx);
@@ -1016,7 +1024,7 @@ fe_status fe_tune(fe_ctx *ctx, fe_elem_type type, const fe_elem_args *a, const f
             for (int pers = 0; pers < 2; ++pers) cands.push_back(Shape{warps * epw, pers, tpe});
     }
     for (const Shape &sh : cands) {
-        if (smem_bytes(type, a, out_mode(o), sh.block) + kStaticSmem > ctx->max_smem_optin) continue;
+        if (smem_bytes(type, a, out_mode(o), sh.block, sh.tpe) + kStaticSmem > ctx->max_smem_optin) continue;
         st = launch_set(ctx, type, a, o, ctx->scratch, s, &sh);  // warm-up
         if (st != FE_OK) break;
         cudaEventRecord(e0, s);
