@@ -132,6 +132,16 @@ FE_HD double fx_double(uint32_t hi, uint32_t lo) {
 // Biased exponent field of |v|.
 FE_HD int fx_exp(double v) { return static_cast<int>((fx_hi(v) >> 20) & 0x7FFu); }
 
+// m 2^-d, d >= 0, rounded down (0 or -1 for d > 63).
+FE_HD int64_t fx_shr(int64_t m, int d) {
+#ifdef __CUDA_ARCH__
+    asm("shr.s64 %0, %0, %1;" : "+l"(m) : "r"(d));   // amounts above 63 count as 63
+    return m;
+#else
+    return m >> (d > 63 ? 63 : d);
+#endif
+}
+
 // v's significand 2^(52 + SH) scaled to an exponent field d above v's own,
 // truncated toward zero: an integer below 2^(53 + SH) in magnitude. Zero (and a
 // subnormal) gives 0 when d >= 64.
@@ -186,10 +196,11 @@ FE_HD double fx_recip(double v, double w) {
 #endif
 }
 
-// Largest exponent of doubles, accumulated over their high words. On the device the
-// words compare as floats' magnitudes (one instruction for two of them, the sign
-// dropped); a word that is a float NaN (|v| >= 2^1017, infinities, NaN) gives NaN,
-// whose exponent field is outside every window.
+FE_HD int fx_maxi(int a, int b) { return a > b ? a : b; }
+// The largest of three doubles' magnitudes by their high words (the first already
+// without its sign). On the device the words compare as floats' magnitudes (one
+// instruction, the signs dropped); a word that is a float NaN (|v| >= 2^1017,
+// infinities, NaN) gives NaN, whose exponent field is outside every window.
 FE_HD uint32_t fx_max3(uint32_t m, uint32_t a, uint32_t b) {
 #ifdef __CUDA_ARCH__
     float r;
@@ -221,23 +232,31 @@ template <class S> FE_HD void fx_quad(const S &s, int j, double v[4]) {
 // as they are in memory, and f (a_s, t) needs nine products, f t being
 // sign(det J) W / 4. Edges are differences in double (as the double form's).
 //
-// False (nothing written) for elements that the double form takes: exponent
-// fields of the edges or of the weighted coefficients outside the windows below
-// (infinities and NaN among them), det J below 2^-20 of
-// |edge| |cofactor| (nearly or exactly degenerate: its sign and the degeneracy
-// test are then those of the double form) or cofactors below 2^-8 of |edge|^2
-// (needles, whose entries would lose relative accuracy).
+// The coordinate axes carry an exponent each (that of the largest edge component
+// along the axis), so that axis-aligned flat or long elements lose nothing: with
+// D = diag(2^X) over the axes' cofactors and t, (a_r, t) = a^_r D and the integers
+// a^_r meet the coefficients D C^ D, which share one exponent per element.
+//
+// False (nothing written) for elements that the double form takes: exponents of
+// the edges or of the results outside the windows below (infinities and NaN among
+// them), det J below 2^-20 of |edge| |cofactor| after that scaling (nearly or
+// exactly degenerate: its sign and the degeneracy test are then those of the
+// double form) or all cofactors below 2^-8 of |edge|^2 (nearly parallel edges).
 struct TetFx {
-    static constexpr int kEdgeWin = 200, kCoefWin = 300;   // exponents, in powers of two around 1
-    static constexpr int kMaxA = 12, kMaxDet = 24;         // largest normalising shifts (2 and 3 of them headroom)
+    static constexpr int kMaxA = 12, kMaxDet = 24;   // largest normalising shifts (3 to 4 of them usual)
+    // Edges within 2^+-80 bound every exponent sum below by |X_i + X_k - xt| <= 330:
+    // results within 2^-700 .. 2^600 (of their last bit) then exclude an infinite or
+    // NaN coefficient (2^1024 and more) and admit any within 2^+-300.
+    static constexpr int kEdgeWin = 80, kLow = -700, kHigh = 600;
+    FE_HD static bool outside(int x) { return static_cast<unsigned>(x - kLow) > static_cast<unsigned>(kHigh - kLow); }
 
-    Fx2 a[3][3];        // cofactor rows 1..3, exponent xa
-    Fx2 t;              // det / 4, exponent xt
+    Fx2 a[3][3];        // cofactor rows 1..3, exponents X[0..2] along the axes
+    Fx2 t;              // det / 4, exponent X[3]
     Fx2 f;              // W / |det|, exponent xf
     int64_t half;       // 2^31 (rounding of sums), from run-time data: see geometry
-    int xa, xt, xf;
+    int X[4], xf;
     bool neg;           // det < 0
-    double vn;          // |det| / 4 / 2^(xt + 60), in [1, 2]
+    double vn;          // |det| / 4 / 2^(X[3] + 60), in [1, 2]
 
     template <class XS> FE_HD bool geometry(const XS &x) {
         double ed[9];
@@ -250,25 +269,25 @@ struct TetFx {
 #else
                 ed[3 * k + i] = x(3 * (k + 1) + i) - x(i);
 #endif
-        uint32_t eb = fx_max3(fx_hi(ed[0]) & 0x7FFFFFFFu, fx_hi(ed[1]), fx_hi(ed[2]));
+        int Ee[3];
 #pragma unroll
-        for (int j = 3; j < 9; j += 2) eb = fx_max3(eb, fx_hi(ed[j]), fx_hi(ed[j + 1]));
-        const int Ee = static_cast<int>(eb >> 20);
-        if (static_cast<unsigned>(Ee - 1023 + kEdgeWin) > 2u * kEdgeWin) return false;
+        for (int i = 0; i < 3; ++i) {
+            Ee[i] = static_cast<int>(fx_max3(fx_hi(ed[i]) & 0x7FFFFFFFu, fx_hi(ed[3 + i]), fx_hi(ed[6 + i])) >> 20);
+            if (static_cast<unsigned>(Ee[i] - 1023 + kEdgeWin) > 2u * kEdgeWin) return false;
+        }
         // 2^31 up to 2^11, not a constant to the compiler: a constant start of a sum
         // of products kept ptxas from fusing the first product's addition
-        half = static_cast<int64_t>(0x80000000u | static_cast<uint32_t>(Ee));
+        half = static_cast<int64_t>(0x80000000u | static_cast<uint32_t>(Ee[0]));
         Fx2 e[3][3], n[3][3];   // edges and their negatives
 #pragma unroll
         for (int k = 0; k < 3; ++k)
 #pragma unroll
             for (int i = 0; i < 3; ++i) {
-                Fx2 v = fx_limbs(fx_from<8>(ed[3 * k + i], Ee - fx_exp(ed[3 * k + i])));
+                Fx2 v = fx_limbs(fx_from<8>(ed[3 * k + i], Ee[i] - fx_exp(ed[3 * k + i])));
                 v.l = v.l > -0x7FFFFFFF ? v.l : -0x7FFFFFFF;   // so that -l exists
                 e[k][i] = v;
                 n[k][i] = {-v.h, -v.l};
             }
-        const int xe = Ee - 1023 - 60;
         int64_t r[3][3];
         uint32_t bits = 0;
 #pragma unroll
@@ -289,23 +308,25 @@ struct TetFx {
         for (int m = 0; m < 3; ++m)
 #pragma unroll
             for (int i = 0; i < 3; ++i) a[m][i] = fx_limbs(static_cast<int64_t>(static_cast<uint64_t>(r[m][i]) << na));
-        xa = 2 * xe + 64 - na;
+        const int xs = Ee[0] + Ee[1] + Ee[2] - 3 * (1023 + 60) + 64 - na;   // exponent of edge x cofactor
+#pragma unroll
+        for (int i = 0; i < 3; ++i) X[i] = xs - (Ee[i] - 1023 - 60);
         const int64_t d = fx_dot3(e[0], a[0], half);
         const int nd = fx_shift(fx_hi_bits(d));
         if (nd > kMaxDet) return false;
         const int64_t dm = static_cast<int64_t>(static_cast<uint64_t>(d) << nd);
         t = fx_limbs(dm);
-        xt = xe + xa + 62 - nd;
+        X[3] = xs + 62 - nd;
         neg = dm < 0;
         vn = fx_to(neg ? -dm : dm, -60);
-        // f = W / |det| = (4/3) / vn 2^(-125 - xt)
+        // f = W / |det| = (4/3) / vn 2^(-125 - X[3])
         const double fd = fx_recip(vn, 4.0 / 3.0);
         f = fx_limbs(fx_from<8>(fd, 1023 - fx_exp(fd)));
-        xf = -125 - xt;
+        xf = -125 - X[3];
         return true;
     }
-    // f a_m in units of 2^(xf + xa + 61): at most (4/3) 2^60 (f t is +-(2/3) 2^60 of
-    // 2^(xf + xt + 61))
+    // f a_m in units of 2^(xf + X[i] + 61): at most (4/3) 2^60 (f t is +-(2/3) 2^60 of
+    // 2^(xf + X[3] + 61))
     FE_HD void scaled(Fx2 fa[3][3]) const {
 #pragma unroll
         for (int m = 0; m < 3; ++m)
@@ -314,15 +335,21 @@ struct TetFx {
     }
 
     // |det J|
-    FE_HD double volume() const { return fx_double(fx_hi(vn) + (static_cast<uint32_t>(xt + 62) << 20), fx_lo(vn)); }
+    FE_HD double volume() const { return fx_double(fx_hi(vn) + (static_cast<uint32_t>(X[3] + 62) << 20), fx_lo(vn)); }
 
     // Laplace kind: A_rs = f a_r . a_s (r, s = 1..3), row and column 0 from the
     // vanishing sums.
     FE_HD void laplace(double A[16]) const {
-        const int xo = xf + 61 + 2 * xa + 64;
+        // the axes' products brought to the largest axis' exponent
+        int xm = X[0] > X[1] ? X[0] : X[1];
+        xm = xm > X[2] ? xm : X[2];
+        const int xo = xf + 61 + 2 * xm + 64;
         int64_t row0[3] = {0, 0, 0};
         Fx2 fa[3][3];
-        scaled(fa);
+#pragma unroll
+        for (int m = 0; m < 3; ++m)
+#pragma unroll
+            for (int i = 0; i < 3; ++i) fa[m][i] = fx_limbs(fx_shr(fx_mul8(f, a[m][i]), 2 * (xm - X[i])));
 #pragma unroll
         for (int r = 0; r < 3; ++r)
 #pragma unroll
@@ -347,60 +374,58 @@ struct TetFx {
         int xo;
     };
     template <bool MASS2, class CS> FE_HD bool columns(const CS &c, Rows &R, double b[4]) const {
-        // exponents of the weighted coefficients: c^{ij} 2^(2 xa), the rest in dt steps
-        const int dt = xt - xa;
-        uint32_t m0 = 0, m1 = 0, m2, mb = 0, md;
+        // exponents of D C^ D (axis 3: t) and of the weighted load coefficients
+        int Ec, Eb;
         {
-            double u[4], v[4];
-            fx_quad(c, 0, u);
-            m2 = fx_hi(u[0]) & 0x7FFFFFFFu;
-            m1 = fx_max3(m1, fx_hi(u[1]), fx_hi(u[2]));
-            fx_quad(c, 4, v);
-            m1 = fx_max3(m1, fx_hi(u[3]), fx_hi(v[0]));
-            m0 = fx_max3(m0, fx_hi(v[1]), fx_hi(v[2]));
-            fx_quad(c, 8, u);
-            m0 = fx_max3(m0, fx_hi(v[3]), fx_hi(u[1]));
-            m0 = fx_max3(m0, fx_hi(u[2]), fx_hi(u[3]));
-            fx_quad(c, 12, v);
-            m1 = fx_max3(m1, fx_hi(u[0]), fx_hi(v[0]));
-            m0 = fx_max3(m0, fx_hi(v[1]), fx_hi(v[2]));
-            m0 = fx_max3(m0, 0u, fx_hi(v[3]));
-            fx_quad(c, 16, u);
-            md = fx_hi(u[0]) & 0x7FFFFFFFu;
-            mb = fx_max3(mb, fx_hi(u[1]), fx_hi(u[2]));
-            mb = fx_max3(mb, 0u, fx_hi(u[3]));
+            double v[4];
+            fx_quad(c, 0, v);
+            Ec = fx_exp(v[0]) + 2 * X[3];
+            int E3 = 0;                         // row and column of t, before its own X[3]
+#pragma unroll
+            for (int j = 0; j < 3; ++j) E3 = fx_maxi(E3, fx_exp(v[j + 1]) + X[j]);
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                fx_quad(c, 4 * (i + 1), v);
+                E3 = fx_maxi(E3, fx_exp(v[0]) + X[i]);
+#pragma unroll
+                for (int j = 0; j < 3; ++j) Ec = fx_maxi(Ec, fx_exp(v[j + 1]) + (X[i] + X[j]));
+            }
+            Ec = fx_maxi(Ec, E3 + X[3]);
+            fx_quad(c, 16, v);
+            Eb = fx_exp(v[0]) + X[3];
+#pragma unroll
+            for (int i = 0; i < 3; ++i) Eb = fx_maxi(Eb, fx_exp(v[i + 1]) + X[i]);
         }
-        const int E0 = static_cast<int>(m0 >> 20), E1 = static_cast<int>(m1 >> 20) + dt, E2 = static_cast<int>(m2 >> 20) + 2 * dt;
-        int Ec = E0 > E1 ? E0 : E1;
-        Ec = Ec > E2 ? Ec : E2;
-        const int Eb0 = static_cast<int>(mb >> 20), Eb1 = static_cast<int>(md >> 20) + dt;
-        int Eb = Eb0 > Eb1 ? Eb0 : Eb1;
+        R.xo = Ec - 1023 - 59 + xf + 189;
+        int xb = Eb - 1023 - 60 - 63 + 61 + 64;
         // outside the window: exact zeros (no operator, no load) are fine
-        if (static_cast<unsigned>(Ec - 1023 + kCoefWin) > 2u * kCoefWin) {
+        if (outside(R.xo)) {
             for (int j = 0; j < 16; ++j)
                 if (c(j) != 0.0) return false;   // NaN compares unequal
-            Ec = 1023;
+            Ec += -R.xo;                         // any exponent in the window: all integers are 0
+            R.xo = 0;
         }
-        if (static_cast<unsigned>(Eb - 1023 + kCoefWin) > 2u * kCoefWin) {
+        if (outside(xb)) {
             for (int j = 16; j < 20; ++j)
                 if (c(j) != 0.0) return false;
-            Eb = 1023;
+            Eb += -xb;
+            xb = 0;
         }
 #ifdef __CUDA_ARCH__
         asm volatile("" ::: "memory");   // read again below: 40 registers less than holding them
 #endif
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            const int w = k == 3 ? dt : 0;
+            const int w = Ec - X[k];
             const int col = k == 3 ? 0 : k + 1;
             Fx2 ck[4];
 #pragma unroll
             for (int i = 0; i < 3; ++i) {
                 const double v = c(4 * (i + 1) + col);
-                ck[i] = fx_limbs(fx_from<7>(v, Ec - w - fx_exp(v)));
+                ck[i] = fx_limbs(fx_from<7>(v, w - X[i] - fx_exp(v)));
             }
             const double v = c(col);
-            int64_t m = fx_from<7>(v, Ec - w - dt - fx_exp(v));
+            int64_t m = fx_from<7>(v, w - X[3] - fx_exp(v));
             if (MASS2 && k == 3) m = fx_mul8(fx_limbs(m), fx_limbs(0x1999999999999999ll));   // 0.8 2^61
             ck[3] = fx_limbs(m);
             FxAcc T{half, 0};
@@ -418,21 +443,19 @@ struct TetFx {
             R.P[0][k] = p0;
             if (k == 3) R.pm = MASS2 ? tk : 0;
         }
-        R.xo = (Ec - 1023 - 59 + 2 * xa) + xf + 189;
         // load vector
         const Fx2 w = fx_limbs(neg ? -0x1555555555555555ll : 0x1555555555555555ll);   // sign(det) W = +-(4/3) 2^60 2^-63
         Fx2 d[3];
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
             const double v = c(17 + i);
-            d[i] = fx_limbs(fx_mul8(fx_limbs(fx_from<8>(v, Eb - fx_exp(v))), w));
+            d[i] = fx_limbs(fx_mul8(fx_limbs(fx_from<8>(v, Eb - X[i] - fx_exp(v))), w));
         }
         const double v0 = c(16);
-        const Fx2 d0 = fx_limbs(fx_mul8(fx_limbs(fx_from<8>(v0, Eb - dt - fx_exp(v0))), w));
+        const Fx2 d0 = fx_limbs(fx_mul8(fx_limbs(fx_from<8>(v0, Eb - X[3] - fx_exp(v0))), w));
         FxAcc T{half, 0};
         T.mul(t, d0);
         int64_t b0 = T.get() * 4;
-        const int xb = (Eb - 1023 - 60 + xa) - 63 + 61 + 64;
 #pragma unroll
         for (int r = 1; r < 4; ++r) {
             FxAcc s = T;

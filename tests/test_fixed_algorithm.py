@@ -82,6 +82,10 @@ def family(name, n=4000):
     x = o + h * (base + jit * rng.uniform(-1, 1, (n, 4, 3)))
     if name == "flat":
         x[:, :, 2] = o[:, :, 2] + 0.05 * (x[:, :, 2] - o[:, :, 2])
+    if name == "thin":
+        x[:, :, 2] = o[:, :, 2] + 1e-3 * (x[:, :, 2] - o[:, :, 2])
+    if name == "long":
+        x[:, :, 1:] = o[:, :, 1:] + 1e-3 * (x[:, :, 1:] - o[:, :, 1:])
     if name == "slivers":
         t = np.exp(rng.uniform(np.log(2e-3), np.log(2e-2), (n, 1)))
         m = x[:, :3].mean(1)
@@ -114,7 +118,7 @@ def rel(v, r):
 
 
 @pytest.mark.parametrize("four", [0, 1])
-@pytest.mark.parametrize("name", ["regular", "structured", "fine", "large", "scales", "flat", "slivers", "inverted",
+@pytest.mark.parametrize("name", ["regular", "structured", "fine", "large", "scales", "flat", "thin", "long", "slivers", "inverted",
                                   "mass", "advection", "wild", "no_load", "no_operator"])
 def test_fixed_point_no_further_than_double(lib, name, four):
     if np.finfo(np.longdouble).eps > 2e-19:
@@ -139,12 +143,13 @@ def test_out_of_window_elements_are_left(lib):
     x[3] = (x[3] - x[3, 0]) * 2.0 ** -300              # below it
     x[4, 2, 1] = np.inf
     x[5, 2, 1] = np.nan
-    x[6, :, 1:] = x[6, :1, 1:] + 1e-5 * (x[6, :, 1:] - x[6, :1, 1:])   # needle
+    s = np.array([0, 1, 2, 3.0])[:, None] * 1e-2
+    x[6] = s + 1e-5 * (x[6] - x[6, :1])                # a needle along (1, 1, 1)
     c[7, 6] = np.inf
     c[8, 0] = np.nan
     c[9, 18] = np.nan
-    c[10, :16] *= 2.0 ** 500
-    c[11, 16:] *= 2.0 ** -700
+    c[10, :16] *= 2.0 ** 700
+    c[11, 16:] *= 2.0 ** -750
     A, b, L, vol, ok = fixed(lib, x, c, 1)
     assert not ok[:7, 0].any() and ok[7:, 0].all()
     assert not ok[7:12, 1].any() and ok[12:, 1].all()
