@@ -9,6 +9,7 @@
 #include "fe_dword.cuh"
 #include "fe_f64int.cuh"
 #include "fe_fixed.cuh"
+#include "fe_fixed_prism.cuh"
 #include "fe_internal.h"
 
 namespace fe {

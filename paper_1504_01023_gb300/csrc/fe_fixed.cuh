@@ -65,15 +65,17 @@ struct FxAcc {
     }
     // in units of 2^64: rounded if mid started at 2^31, else truncated
     FE_HD int64_t get() const { return hh + (mid >> 32); }
-    // in units of 2^61, truncated (one product of normalised operands)
-    FE_HD int64_t get8() const { return (hh << 3) + (mid >> 29); }
+    // in units of 2^(64 - N), truncated unless mid started at 2^(31 - N)
+    template <int N> FE_HD int64_t get() const {
+        return static_cast<int64_t>(static_cast<uint64_t>(hh) << N) + (mid >> (32 - N));
+    }
 };
 
-// a b in units of 2^61
-FE_HD int64_t fx_mul8(Fx2 a, Fx2 b) {
-    FxAcc s{0, 0};
+// a b in units of 2^61 (rounded with round = 2^28)
+FE_HD int64_t fx_mul8(Fx2 a, Fx2 b, int64_t round = 0) {
+    FxAcc s{round, 0};
     s.mul(a, b);
-    return s.get8();
+    return s.get<3>();
 }
 FE_HD int64_t fx_dot3(const Fx2 a[3], const Fx2 b[3], int64_t half) {
     FxAcc s{half, 0};
@@ -83,6 +85,8 @@ FE_HD int64_t fx_dot3(const Fx2 a[3], const Fx2 b[3], int64_t half) {
     return s.get();
 }
 
+FE_HD int fx_maxi(int a, int b) { return a > b ? a : b; }
+FE_HD int fx_mini(int a, int b) { return a < b ? a : b; }
 // Leading zeros of a 32-bit word (32 for 0).
 FE_HD int fx_clz(uint32_t v) {
 #ifdef __CUDA_ARCH__
@@ -196,7 +200,6 @@ FE_HD double fx_recip(double v, double w) {
 #endif
 }
 
-FE_HD int fx_maxi(int a, int b) { return a > b ? a : b; }
 // The largest of three doubles' magnitudes by their high words (the first already
 // without its sign). On the device the words compare as floats' magnitudes (one
 // instruction, the signs dropped); a word that is a float NaN (|v| >= 2^1017,

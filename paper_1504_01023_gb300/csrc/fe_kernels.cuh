@@ -289,24 +289,37 @@ template <int KIND, int QUAD, int CPQ> struct ElemMath<TET, KIND, DWORD, QUAD, C
 // edge vectors.
 // The half of a prism's A^e and b^e that lane `part` of a pair writes: entry
 // pair_entry(j, part) of A^e (row-major) in Ah[j], entry pair_b_entry(j, part) of
-// b^e in bh[j]. Laplace: entries 2j + part, picked from the whole A^e and b^e that
-// both lanes hold. Generic: lane 0 the diagonal blocks (bottom-bottom, top-top) of
-// A^e and b_0..2, lane 1 the off-diagonal blocks and b_3..5, as pair_blocks leaves
-// them in A[0..17] and b[0..2].
-template <int KIND> __device__ __forceinline__ int pair_entry(int j, int part) {
-    if constexpr (KIND == GENERIC) {
+// b^e in bh[j]. By blocks (generic kind, and the FP64 form): lane 0 the diagonal
+// blocks (bottom-bottom, top-top) of A^e and b_0..2, lane 1 the off-diagonal blocks
+// and b_3..5, as pair_blocks leaves them in A[0..17] and b[0..2]. Else (Laplace):
+// entries 2j + part, picked from the whole A^e and b^e that both lanes hold.
+template <int KIND, int PREC> __host__ __device__ constexpr bool pair_by_blocks() { return KIND == GENERIC || PREC == FP64; }
+// Two threads per element in block fixed point keep 60 values per thread: generic
+// kind with per-point coefficients in the coefficients' own shared memory, with
+// per-element coefficients in 960 bytes per element behind the tile's inputs.
+template <int KIND, int PREC, int CPQ> __host__ __device__ constexpr bool pair_scratch() {
+    return KIND == GENERIC && PREC == FP64 && CPQ == 0;
+}
+template <int KIND, int PREC> __device__ __forceinline__ int pair_entry(int j, int part) {
+    if constexpr (pair_by_blocks<KIND, PREC>()) {
         const int blk = j / 9, k = (j % 9) / 3, kk = j % 3;
         return 6 * (k + 3 * blk) + kk + 3 * (blk ^ part);
     } else {
         return 2 * j + part;
     }
 }
-template <int KIND> __device__ __forceinline__ int pair_b_entry(int j, int part) {
-    return KIND == GENERIC ? 3 * part + j : 2 * j + part;
+template <int KIND, int PREC> __device__ __forceinline__ int pair_b_entry(int j, int part) {
+    return pair_by_blocks<KIND, PREC>() ? 3 * part + j : 2 * j + part;
 }
-template <int KIND, class T>
+template <int KIND, int PREC, class T>
 __device__ __forceinline__ void pick_half(const T A[36], const T b[6], T Ah[18], T bh[3], int part) {
-    if constexpr (KIND == GENERIC) {
+    if constexpr (KIND == POISSON && PREC == FP64) {
+#pragma unroll
+        for (int j = 0; j < 18; ++j)
+            Ah[j] = part ? A[pair_entry<KIND, PREC>(j, 1)] : A[pair_entry<KIND, PREC>(j, 0)];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) bh[j] = part ? b[3 + j] : b[j];
+    } else if constexpr (KIND == GENERIC) {
 #pragma unroll
         for (int j = 0; j < 18; ++j) Ah[j] = A[j];
 #pragma unroll
@@ -814,6 +827,13 @@ template <int KIND, int PREC, int CPQ> struct PrismMath {
     }
 };
 
+// An accessor's values from `off` on.
+template <class S> struct OffSrc {
+    const S &s;
+    int off;
+    __device__ __forceinline__ double operator()(int j) const { return s(off + j); }
+};
+
 template <int KIND, int CPQ> struct ElemMath<PRISM, KIND, FP64, Q_PRISM6, CPQ> {
     template <class XS> __device__ __forceinline__ static void rel(const XS &x, V3<double> r[6]) {
         const V3<double> x0 = {x(0), x(1), x(2)};
@@ -838,22 +858,69 @@ template <int KIND, int CPQ> struct ElemMath<PRISM, KIND, FP64, Q_PRISM6, CPQ> {
         }
         return fl;
     }
-    // Two threads per element: this lane's zeta level; the lane's half out (pick_half).
-    template <class XS, class CS>
-    __device__ __forceinline__ static uint8_t run_pair(const XS &x, const CS &c, double Ah[18], double bh[3], bool &poor,
-                                                       int part, unsigned mask) {
+    // Two threads per element: this lane's zeta level in block fixed point (PrismFx);
+    // each lane forms its half of A^e and b^e from both levels' sums (pair_entry). A
+    // pair outside the fixed-point windows takes the double pipe.
+    // scratch: 60 values of this lane's (generic kind; may be its coefficients'
+    // own memory), xg, cg: the element's inputs in global memory.
+    template <class XS, class CS, class XG, class CG>
+    __device__ __forceinline__ static uint8_t run_pair(const XS &x, const CS &c, const XG &xg, const CG &cg,
+                                                       double *scratch, double Ah[18], double bh[3], bool &poor, int part,
+                                                       unsigned mask) {
+        constexpr int NP = CPQ ? 3 : 1, NCP = KIND == POISSON ? 1 : 20;   // points with coefficients of their own
+        const OffSrc<CS> cl{c, CPQ ? NP * NCP * part : 0};
+        PrismFx P;
+        P.v = reinterpret_cast<int64_t *>(scratch);
+        uint32_t b12, b3;
+        P.begin(x, part, b12, b3);
+        b12 |= __shfl_xor_sync(mask, b12, 1);
+        b3 |= __shfl_xor_sync(mask, b3, 1);
+        uint32_t d = P.set_a(b12, b3);
+        P.set_det(d | __shfl_xor_sync(mask, d, 1));
+        P.template exponents<KIND>(cl, NP);
+#pragma unroll
+        for (int j = KIND == POISSON ? 5 : 0; j < 6; ++j) P.En[j] = max(P.En[j], __shfl_xor_sync(mask, P.En[j], 1));
+        P.template common_exponents<KIND>();
+        P.template set_exponents<KIND>(cl, NP);
+#pragma unroll 1
+        for (int t = 0; t < 3; ++t) {   // rolled: unrolled, the kernel (105 KB) left the instruction cache
+            int T12, T3;
+            P.template products<KIND>(cl, CPQ ? NCP : 0, t, T12, T3);
+            if (t == 0) {
+                T12 = max(T12, __shfl_xor_sync(mask, T12, 1));
+                P.set_products(T12, max(T3, __shfl_xor_sync(mask, T3, 1)));
+            }
+            P.template gamma<KIND>(t);
+        }
+        P.template sums<KIND>();
+        P.template align<KIND>(min(P.lza, __shfl_xor_sync(mask, P.lza, 1)), min(P.lzb, __shfl_xor_sync(mask, P.lzb, 1)));
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+            long long X, Y, U, V;
+            P.blocks(part, i, X, Y, U, V);
+            const long long p = (part ? U : X) + __shfl_xor_sync(mask, part ? X : U, 1);
+            const long long q = (part ? V : Y) + __shfl_xor_sync(mask, part ? Y : V, 1);
+            Ah[i] = P.out_a(p + q);
+            Ah[9 + i] = P.out_a(p - q);
+        }
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            long long X, Y;
+            P.loads(part, k, X, Y);
+            const long long p = X + __shfl_xor_sync(mask, X, 1), q = Y + __shfl_xor_sync(mask, Y, 1);
+            bh[k] = P.out_b(part ? p - q : p + q);
+        }
+        poor = false;
+        const bool neg = pair_any(P.neg, mask);
+        if (!pair_any(!P.ok, mask)) return neg ? 2 : 0;
+        // the double pipe, from the inputs in global memory; shuffles within the pair alone
+        const unsigned pm = 3u << ((threadIdx.x & 31u) & ~1u);
         V3<double> r[6];
-        rel(x, r);
+        rel(xg, r);
         double A[36], b[6];
         bool sp = false;
-        uint8_t fl = PrismMath<KIND, FP64, CPQ>::template qloop<2>(r, c, A, b, poor, sp, part, mask);
-        if (sp) {   // both lanes of the pair: their shuffles within the pair alone
-            asm volatile("" ::: "memory");
-            rel(x, r);
-            const unsigned pm = 3u << ((threadIdx.x & 31u) & ~1u);
-            fl = PrismMath<KIND, FP64, CPQ>::template qloop<2, true>(r, c, A, b, poor, sp, part, pm);
-        }
-        pick_half<KIND>(A, b, Ah, bh, part);
+        const uint8_t fl = PrismMath<KIND, FP64, CPQ>::template qloop<2, true>(r, cg, A, b, poor, sp, part, pm);
+        pick_half<KIND, FP64>(A, b, Ah, bh, part);
         return fl;
     }
 };
@@ -887,7 +954,7 @@ template <int KIND, int CPQ> struct ElemMath<PRISM, KIND, MIXED, Q_PRISM6, CPQ> 
         float A[36], b[6];
         bool sp;   // set by the FP64 form only
         const uint8_t fl = PrismMath<KIND, MIXED, CPQ>::template qloop<2>(r, c, A, b, poor, sp, part, mask);
-        pick_half<KIND>(A, b, Ah, bh, part);
+        pick_half<KIND, MIXED>(A, b, Ah, bh, part);
         return fl;
     }
     // Flagged element: Jacobian terms in double at every point, narrowed to float.
@@ -967,7 +1034,7 @@ template <int KIND, int CPQ> struct ElemMath<PRISM, KIND, DWORD, Q_PRISM6, CPQ> 
         bool sp;   // set by the FP64 form only
         const uint8_t fl = PrismMath<KIND, DWORD, CPQ>::template qloop<2>(r, cd, Ad, bd, poor, sp, part, mask);
         DW Adh[18], bdh[3];
-        pick_half<KIND>(Ad, bd, Adh, bdh, part);
+        pick_half<KIND, DWORD>(Ad, bd, Adh, bdh, part);
         // the group tests on the sums over both halves (the same on both lanes); the
         // shuffles run on every lane of `mask`, whatever the lane's flags
         const float sa = dw_abs_sum<18>(Adh), sb = dw_abs_sum<3>(bdh);
@@ -1693,6 +1760,13 @@ __device__ __forceinline__ bool process_tile(const ElemParams &p, int64_t e0, in
             const SmemSrc<double> xs{INL == SOA ? sX + tid : sX + tid * NX, INL == SOA ? B : 1};
             if constexpr (TPE == 1)
                 fl = run_elem<ET, KIND, PREC, QUAD, CPQ>(xs, cs, fn, A, b, poor);
+            else if constexpr (TPE == 2 && PREC == FP64)
+                fl = ElemMath<ET, KIND, PREC, QUAD, CPQ>::run_pair(
+                    xs, cs, Src<AOS, double>{X + e * NX, 0}, Src<AOS, double>{C + e * NC, 0},
+                    pair_scratch<KIND, PREC, CPQ>()
+                        ? reinterpret_cast<double *>(smem + SM::x_bytes(B) + SM::c_bytes(B)) + (2 * tid + sub) * 60
+                        : sC + tid * NC + (CPQ ? NC / 2 : 0) * sub,
+                    A, b, poor, sub, pmask);
             else if constexpr (TPE == 2)
                 fl = ElemMath<ET, KIND, PREC, QUAD, CPQ>::run_pair(xs, cs, A, b, poor, sub, pmask);
             else if constexpr (ET == TET && TPE == 16)
@@ -1715,9 +1789,9 @@ __device__ __forceinline__ bool process_tile(const ElemParams &p, int64_t e0, in
     __syncthreads();   // every input read: the output records reuse the same shared memory
     if (TPE == 2 && active) {
 #pragma unroll
-        for (int j = 0; j < NA / TPE; ++j) sA[tid * NAO + pair_entry<KIND>(j, sub)] = A[j];
+        for (int j = 0; j < NA / TPE; ++j) sA[tid * NAO + pair_entry<KIND, PREC>(j, sub)] = A[j];
 #pragma unroll
-        for (int j = 0; j < NS / TPE; ++j) sB[tid * NS + pair_b_entry<KIND>(j, sub)] = b[j];
+        for (int j = 0; j < NS / TPE; ++j) sB[tid * NS + pair_b_entry<KIND, PREC>(j, sub)] = b[j];
     }
     if (TPE == NS && TPE > 2 && active) {
 #pragma unroll
@@ -1856,8 +1930,7 @@ template <int KIND, int QUAD, int CPQ, int INL, int OUTL> const void *dw_tet_ker
 // tiles of blockDim.x / 2 elements, grid-stride over tiles.
 // ---------------------------------------------------------------------------
 template <int KIND, int PREC, int CPQ>
-__global__ void __launch_bounds__(256)
-    pair_kernel(const ElemParams p, const __grid_constant__ TmaMaps tm, const __grid_constant__ CoefFn fn) {
+__device__ __forceinline__ void pair_tiles(const ElemParams &p, const TmaMaps *tm, const CoefFn *fn) {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ uint64_t bar;
     if (threadIdx.x == 0) {
@@ -1875,10 +1948,27 @@ __global__ void __launch_bounds__(256)
         }
         const int64_t e0 = tile * B;
         const int nb = static_cast<int>(p.n - e0 < B ? p.n - e0 : B);
-        if (!process_tile<PRISM, KIND, PREC, Q_PRISM6, CPQ, AOS, AOS, 2>(p, e0, nb, smem, &bar, phase, &tm, &fn))
+        if (!process_tile<PRISM, KIND, PREC, Q_PRISM6, CPQ, AOS, AOS, 2>(p, e0, nb, smem, &bar, phase, tm, fn))
             return;
     }
     if (threadIdx.x < 32) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+}
+template <int KIND, int PREC, int CPQ>
+__global__ void __launch_bounds__(256)
+    pair_kernel(const ElemParams p, const __grid_constant__ TmaMaps tm, const __grid_constant__ CoefFn fn) {
+    pair_tiles<KIND, PREC, CPQ>(p, &tm, &fn);
+}
+// The FP64 form in block fixed point (PrismFx). Bound by issue and by the latency of
+// its chains at 8 to 16 warps per SM (6,500 instructions per thread, half of them
+// 32-bit integer operations; 51 double instructions against about 1,500 per element
+// in the double form, which the double pipe bounded at 0.89 of its rate). 400,000
+// prisms with per-point coefficients: 0.376 -> 1.29 Gelem/s (128 registers 1.09, 168
+// 1.25, 200 1.29, 255 1.28), per-element 1.36 (168 registers 1.29, 255 1.36),
+// Laplace 1.04 -> 2.80 (96 registers 2.76, 128 2.80, 168 2.64).
+template <int KIND, int CPQ>
+__global__ void __launch_bounds__(256) __maxnreg__(KIND == POISSON ? 128 : (CPQ ? 200 : 255))
+    pair_kernel_f64(const ElemParams p, const __grid_constant__ TmaMaps tm, const __grid_constant__ CoefFn fn) {
+    pair_tiles<KIND, FP64, CPQ>(p, &tm, &fn);
 }
 
 // ---------------------------------------------------------------------------

@@ -184,6 +184,9 @@ static int64_t smem_bytes(fe_elem_type type, const fe_elem_args *a, int outl, in
     const int64_t in = geo + r16(int64_t(B) * nc * cs),
                   out = r16(int64_t(B) * na_out(type, outl) * cs) + r16(int64_t(B) * ns * cs);
     if (outl == kOutApply) return in;  // matrix-free: results leave from registers
+    // the two-thread FP64 form's scratch behind the inputs (pair_scratch)
+    if (tpe == 2 && a->prec == FE_FP64 && a->kind == FE_GENERIC && a->coef_mode == FE_COEF_PER_ELEMENT)
+        return std::max(in + int64_t(B) * 960, out);
     return in > out ? in : out;
 }
 
