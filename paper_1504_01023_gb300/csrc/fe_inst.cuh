@@ -3,9 +3,19 @@
 #pragma once
 #include "fe_stream.cuh"
 
+namespace fe {
+// The tile kernel, or null where plane_kernel always runs (plane_always).
+template <int ET, int KIND, int PREC, int QUAD, int CPQ, int INL, int OUTL> const void *tile_kernel() {
+    if constexpr (INL == SOA && out_soa(OUTL) && plane_always(ET, KIND, PREC, CPQ))
+        return nullptr;
+    else
+        return reinterpret_cast<const void *>(&elem_kernel<ET, KIND, PREC, QUAD, CPQ, INL, OUTL>);
+}
+}  // namespace fe
+
 #define FE_ELEM_CASE(ET, PREC, QUAD, KD, CP, IL, OL)                                  \
     if (kind == KD && cpq == CP && inl == IL && outl == OL)                          \
-        return reinterpret_cast<const void *>(&fe::elem_kernel<ET, KD, PREC, QUAD, CP, IL, OL>);
+        return fe::tile_kernel<ET, KD, PREC, QUAD, CP, IL, OL>();
 // FP64 tetrahedra: the warp-at-a-time kernel or the register-capped tile kernel
 // (f64_tet_kernel).
 #define FE_F64T_CASE(ET, PREC, QUAD, KD, CP, IL, OL)                                  \
@@ -14,6 +24,9 @@
 // per-element coefficients (dw_tet_kernel).
 #define FE_DWT_CASE(ET, PREC, QUAD, KD, CP, IL, OL)                                   \
     if (kind == KD && cpq == CP && inl == IL && outl == OL) return fe::dw_tet_kernel<KD, QUAD, CP, IL, OL>();
+#define FE_PLANE_CASE(ET, PREC, QUAD, KD, CP, IL, OL)                                 \
+    if (kind == KD && prec == PREC && quad == QUAD && cpq == CP && outl == OL)       \
+        return reinterpret_cast<const void *>(&fe::plane_kernel<ET, KD, PREC, QUAD, CP, OL>);
 #define FE_FIX_CASE(ET, PREC, QUAD, KD, CP, IL, OL)                                   \
     if (kind == KD && cpq == CP && inl == IL && outl == OL)                          \
         return reinterpret_cast<const void *>(&fe::fixup_kernel<ET, KD, PREC, QUAD, CP, IL, OL>);
@@ -25,6 +38,12 @@
     M(__VA_ARGS__, 1, 0, 0, 1) M(__VA_ARGS__, 1, 0, 1, 0) M(__VA_ARGS__, 1, 0, 1, 1)  \
     M(__VA_ARGS__, 1, 1, 0, 0) M(__VA_ARGS__, 1, 1, 0, 1) M(__VA_ARGS__, 1, 1, 1, 0)  \
     M(__VA_ARGS__, 1, 1, 1, 1)
+
+// Plane-major in and out: kind x coefficient mode, and the packed output of the
+// Laplace kind.
+#define FE_PLANE6(M, ...)                                                             \
+    M(__VA_ARGS__, 0, 0, 0, 0) M(__VA_ARGS__, 0, 1, 0, 0) M(__VA_ARGS__, 1, 0, 0, 0)  \
+    M(__VA_ARGS__, 1, 1, 0, 0) M(__VA_ARGS__, 0, 0, 0, 3) M(__VA_ARGS__, 0, 1, 0, 3)
 
 // The eight (coefficient mode, input layout, output layout) combinations of one kind.
 #define FE_ALL8(M, KD, ...)                                                           \

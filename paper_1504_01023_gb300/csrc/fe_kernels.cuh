@@ -2222,12 +2222,18 @@ __device__ __forceinline__ void fixup_element(const ElemParams &p, int64_t e, co
     if (p.flags) p.flags[e] = fl;
 }
 
-// Fix-up kernel of one call: grid-stride over the list written by the main kernel.
+// Fix-up kernel of one call: the list written by the main kernel, 32 entries per warp,
+// consecutive groups of 32 to different blocks, so that a short list spreads over
+// the SMs' double pipes (4,000 flagged generic tetrahedra of 400,000: 14.2 us with a
+// block's 256 threads on consecutive entries, all on 16 SMs).
 template <int ET, int KIND, int PREC, int QUAD, int CPQ, int INL, int OUTL>
 __global__ void __launch_bounds__(256) fixup_kernel(const ElemParams p, const __grid_constant__ CoefFn fn) {
     const unsigned cnt = *p.fix_count;
     const unsigned n = cnt < p.fix_cap ? cnt : p.fix_cap;
-    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    const unsigned lane = threadIdx.x & 31u, warps = blockDim.x >> 5;
+    for (unsigned g = (threadIdx.x >> 5) * gridDim.x + blockIdx.x; g * 32u < n; g += warps * gridDim.x) {
+        const unsigned i = g * 32u + lane;
+        if (i >= n) continue;
         const int64_t e = static_cast<int64_t>(p.fix_list[i] & ((1ull << 40) - 1));
         if (e >= p.n) {
             atomicOr(p.status, ST_BAD_TILE);

@@ -90,7 +90,10 @@ extern "C" fe_status fe_integrate_tet_noalloc(const fe_elem_args *args, const fe
     if (st != FE_OK) return st;
 
     const int cpq = args->coef_mode == FE_COEF_PER_QPOINT;
-    const void *k = kernel_tet_mixed(args->kind, args->quad, cpq, args->coords_layout, out->layout);
+    // plane-major in and out: straight from and to global memory (no tensor maps here)
+    const bool planes = args->coords_layout == FE_LAYOUT_SOA && out->layout == FE_LAYOUT_SOA;
+    const void *k = planes ? kernel_plane_tet(args->kind, FE_FP32_MIXED, args->quad, cpq, SOA)
+                           : kernel_tet_mixed(args->kind, args->quad, cpq, args->coords_layout, out->layout);
     const void *fk = kernel_fixup_tet(args->kind, args->quad, cpq, args->coords_layout, out->layout);
     if (!k || !fk) return set_error(nullptr, FE_ERR_UNSUPPORTED, "no kernel for this combination");
 
@@ -99,7 +102,7 @@ extern "C" fe_status fe_integrate_tet_noalloc(const fe_elem_args *args, const fe
     const int nc = nc_of(FE_TET, args);
     auto r16 = [](int64_t v) { return (v + 15) / 16 * 16; };
     const int64_t smem_in = int64_t(B) * 12 * 8 + r16(int64_t(B) * nc * 4), smem_out = r16(int64_t(B) * 16 * 4) + r16(int64_t(B) * 4 * 4);
-    const int64_t smem = smem_in > smem_out ? smem_in : smem_out;
+    const int64_t smem = planes ? 0 : (smem_in > smem_out ? smem_in : smem_out);
     // raise the kernel's dynamic shared-memory limit if needed, never lower it,
     // through the same record as the other entry points that launch this kernel
     st = set_smem_attr(nullptr, k, smem);

@@ -1,0 +1,75 @@
+// Plane-major inputs and outputs: one element per thread straight between global
+// memory and registers.
+#pragma once
+#include "fe_kernels.cuh"
+
+namespace fe {
+
+// Plane values through the read-only path (read again by forms that scan the
+// coefficients first: the second read hits L1).
+template <class T> struct PlaneSrc {
+    const T *base;
+    int64_t stride;
+    __device__ __forceinline__ T operator()(int j) const { return __ldg(base + j * stride); }
+};
+
+// Scalar j of a warp's 32 elements is one contiguous run of its plane, so loads and
+// stores are coalesced whatever the planes' alignment and pitch, every load of a
+// thread is in flight at once and no block barrier separates them from the
+// arithmetic. skip_mod as for elem_tiles: tiles of blockDim elements.
+template <int ET, int KIND, int PREC, int QUAD, int CPQ, int OUTL>
+__device__ __forceinline__ void plane_elems(const ElemParams &p, const CoefFn *fn) {
+    using CF = ElemCfg<ET, KIND, PREC, QUAD, CPQ>;
+    using CT = typename CF::CT;
+    constexpr int NS = CF::NS, NX = CF::NX, NA = CF::NA, NC = CF::NC;
+    // coefficient planes up to 80 bytes per element are read ahead into registers
+    constexpr bool kCoefRegs = NC * sizeof(CT) <= 80;
+    const CT *C = static_cast<const CT *>(p.C);
+    CT *Aout = static_cast<CT *>(p.A);
+    CT *Bout = static_cast<CT *>(p.B);
+    const int64_t ntiles = (p.n + blockDim.x - 1) / blockDim.x;
+    for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+        if (p.skip_mod > 0 && tile % p.skip_mod == 0) {   // injected fault: no load, no store
+            if (threadIdx.x == 0) atomicOr(p.status, ST_SKIPPED_TILES);
+            continue;
+        }
+        const int64_t e = tile * blockDim.x + threadIdx.x;
+        const bool active = e < p.n;
+        bool poor = false;
+        if (active) {
+            double xr[NX];
+#pragma unroll
+            for (int j = 0; j < NX; ++j) xr[j] = ld_stream(p.X + j * p.xs + e);
+            CT A[NA], b[NS];
+            uint8_t fl;
+            if constexpr (kCoefRegs) {
+                CT cr[NC];
+#pragma unroll
+                for (int j = 0; j < NC; ++j) cr[j] = ld_stream(C + j * p.cs + e);
+                fl = run_elem<ET, KIND, PREC, QUAD, CPQ>(RegSrc<double>{xr}, RegSrc<CT>{cr}, fn, A, b, poor);
+            } else {
+                fl = run_elem<ET, KIND, PREC, QUAD, CPQ>(RegSrc<double>{xr}, PlaneSrc<CT>{C + e, p.cs}, fn, A, b, poor);
+            }
+            if (PREC != FP64 && poor) fl |= 1;
+            if (p.flags) p.flags[e] = fl;
+#pragma unroll
+            for (int r = 0; r < NS; ++r)
+#pragma unroll
+                for (int s = out_packed(OUTL) ? r : 0; s < NS; ++s) {
+                    const int ko = out_packed(OUTL) ? packed_index(NS, r, s) : r * NS + s;
+                    st_stream(Aout + ko * p.os + e, A[r * NS + s]);
+                }
+#pragma unroll
+            for (int k = 0; k < NS; ++k) st_stream(Bout + k * p.os + e, b[k]);
+        }
+        if (PREC != FP64) append_fixup(p, active && poor, e);
+    }
+}
+
+template <int ET, int KIND, int PREC, int QUAD, int CPQ, int OUTL>
+__global__ void __launch_bounds__(ET == TET && PREC != DWORD ? 512 : 256)
+    plane_kernel(const ElemParams p, const __grid_constant__ TmaMaps, const __grid_constant__ CoefFn fn) {
+    plane_elems<ET, KIND, PREC, QUAD, CPQ, OUTL>(p, &fn);
+}
+
+}  // namespace fe

@@ -141,6 +141,11 @@ static const void *main_kernel(fe_elem_type type, const fe_elem_args *a, int out
     return nullptr;
 }
 
+static const void *plane_kernel(fe_elem_type type, const fe_elem_args *a, int outl) {
+    return type == FE_TET ? kernel_plane_tet(a->kind, a->prec, a->quad, cpq_of(a), outl)
+                          : kernel_plane_prism(a->kind, a->prec, a->quad, cpq_of(a), outl);
+}
+
 static const void *fix_kernel(fe_elem_type type, const fe_elem_args *a, int outl) {
     const int cpq = cpq_of(a);
     if (a->ordering) return kernel_fixup_study(type, a->kind, a->quad, cpq, a->ordering);
@@ -174,11 +179,11 @@ static bool stream_ok(fe_elem_type type, const fe_elem_args *a, int outl) {
            (cpq == 0 || (cpq == 1 && a->kind == FE_POISSON));
 }
 
-static int64_t smem_bytes(fe_elem_type type, const fe_elem_args *a, int outl, int B, int tpe) {
+static int64_t smem_bytes(fe_elem_type type, const fe_elem_args *a, int outl, int B, int tpe, bool stream = false) {
     // tetrahedra with a node table read straight from global memory (gather_kernel)
     if (a->coords_layout == FE_LAYOUT_INDEXED && type == FE_TET) return 0;
     const int ns = ns_of(type), nc = nc_of(type, a), cs = csize(a->prec);
-    if (tpe == 1 && stream_ok(type, a, outl)) return int64_t(B) * (96 + 8 * nc);   // results leave from registers
+    if (stream) return int64_t(B) * (96 + 8 * nc);   // results leave from registers
     auto r16 = [](int64_t v) { return (v + 15) / 16 * 16; };
     const int64_t geo = a->coords_layout == FE_LAYOUT_INDEXED ? r16(int64_t(B) * ns * 4) : int64_t(B) * 3 * ns * 8;
     const int64_t in = geo + r16(int64_t(B) * nc * cs),
@@ -284,7 +289,7 @@ static bool encode_planes(void *out, bool dbl, const void *base, uint64_t n, uin
 }
 
 fe_status launch_set(fe_ctx *ctx, fe_elem_type type, const fe_elem_args *a, const fe_out *o, Scratch &s, cudaStream_t st,
-                     const Shape *force, const void *x) {
+                     const Shape *force, const void *x, bool mapped) {
     if (a->n_elem == 0) return FE_OK;
     const int outl = out_mode(o);
     Shape sh = default_shape(type);
@@ -294,25 +299,8 @@ fe_status launch_set(fe_ctx *ctx, fe_elem_type type, const fe_elem_args *a, cons
         auto it = ctx->shapes.find(shape_key(type, a, o));
         if (it != ctx->shapes.end()) sh = it->second;
     }
-    const void *k = main_kernel(type, a, outl, sh.tpe);
-    if (!k) return set_error(ctx, FE_ERR_UNSUPPORTED, "no kernel for this combination");
     const int threads = shape_threads(sh.block, sh.tpe);
     if (!threads) return set_error(ctx, FE_ERR_INVALID_ARG, "bad launch shape");
-    const int64_t smem = smem_bytes(type, a, outl, sh.block, sh.tpe);
-    if (smem + kStaticSmem > ctx->max_smem_optin)
-        return set_error(ctx, FE_ERR_UNSUPPORTED, "shared memory of this launch shape too large");
-    {
-        fe_status e = set_smem_attr(ctx, k, smem);
-        if (e != FE_OK) return e;
-    }
-    const int64_t ntiles = (a->n_elem + sh.block - 1) / sh.block;
-    int64_t grid = ntiles;
-    if (sh.persistent) {
-        int per_sm = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, size_t(smem));
-        grid = std::min<int64_t>(ntiles, int64_t(std::max(per_sm, 1)) * ctx->sms);
-    }
-    grid = std::min<int64_t>(grid, 0x7FFFFFFF);
 
     ElemParams p{};
     p.n = a->n_elem;
@@ -328,6 +316,51 @@ fe_status launch_set(fe_ctx *ctx, fe_elem_type type, const fe_elem_args *a, cons
     p.conn = a->coords_layout == FE_LAYOUT_INDEXED ? a->conn : nullptr;
     p.n_nodes = a->coords_layout == FE_LAYOUT_INDEXED ? a->n_nodes : 0;
     p.xv = x;
+    // plane-major tiles of up to 256 elements move as 2-D tensor copies; plane-major
+    // sets that cannot, or whose form gains nothing from them, run straight from and
+    // to global memory
+    TmaMaps tm;
+    memset(&tm, 0, sizeof tm);
+    const bool soa_in = a->coords_layout == FE_LAYOUT_SOA, soa_out = o->layout == FE_LAYOUT_SOA;
+    bool planes = soa_in && soa_out && plane_always(type, a->kind, a->prec, cpq_of(a));
+    if (!planes && sh.block <= 256) {
+        const int ns = ns_of(type), nc = nc_of(type, a);
+        const bool dbl = a->prec != FE_FP32_MIXED;
+        const uint64_t cs = dbl ? 8 : 4;
+        if (soa_in)
+            p.tma_in = encode_planes(tm.x, true, a->coords, uint64_t(a->n_elem), 3 * ns, uint64_t(p.xs) * 8, sh.block) &&
+                       encode_planes(tm.c, dbl, a->coefs, uint64_t(a->n_elem), nc, uint64_t(p.cs) * cs, sh.block);
+        if (soa_out)
+            p.tma_out = encode_planes(tm.a, dbl, o->A, uint64_t(a->n_elem), na_out(type, outl), uint64_t(p.os) * cs,
+                                      sh.block) &&
+                        encode_planes(tm.b, dbl, o->b, uint64_t(a->n_elem), ns, uint64_t(p.os) * cs, sh.block);
+    }
+    planes = planes || (soa_in && soa_out && !(p.tma_in && p.tma_out));
+
+    // FP64 tetrahedra in host memory take the tile kernel: its bulk stores cross the
+    // host link in long runs, the warp-at-a-time kernel's 32-byte ones do not (6M
+    // generic, in and out over the link: 7.85 against 10.1 ms)
+    const bool stream = sh.tpe == 1 && !mapped && stream_ok(type, a, outl);
+    const void *k = planes                                                   ? plane_kernel(type, a, outl)
+                    : !stream && sh.tpe == 1 && stream_ok(type, a, outl)     ? kernel_tet_fp64_tile(a->kind, a->quad, cpq_of(a))
+                                                                             : main_kernel(type, a, outl, sh.tpe);
+    if (!k) return set_error(ctx, FE_ERR_UNSUPPORTED, "no kernel for this combination");
+    const int64_t smem = planes ? 0 : smem_bytes(type, a, outl, sh.block, sh.tpe, stream);
+    if (smem + kStaticSmem > ctx->max_smem_optin)
+        return set_error(ctx, FE_ERR_UNSUPPORTED, "shared memory of this launch shape too large");
+    {
+        fe_status e = set_smem_attr(ctx, k, smem);
+        if (e != FE_OK) return e;
+    }
+    const int64_t ntiles = (a->n_elem + sh.block - 1) / sh.block;
+    int64_t grid = ntiles;
+    if (sh.persistent) {
+        int per_sm = 0;
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, size_t(smem));
+        grid = std::min<int64_t>(ntiles, int64_t(std::max(per_sm, 1)) * ctx->sms);
+    }
+    grid = std::min<int64_t>(grid, 0x7FFFFFFF);
+
     if (ctx->skip_launches.load() > 0 && !force) {   // injected fault: this launch skips tiles
         if (ctx->skip_launches.fetch_sub(1) > 0) p.skip_mod = ctx->skip_mod;
     }
@@ -345,22 +378,6 @@ fe_status launch_set(fe_ctx *ctx, fe_elem_type type, const fe_elem_args *a, cons
         if (e != FE_OK) return e;
     }
     p.status = s.status;
-
-    // plane-major tiles of up to 256 elements move as 2-D tensor copies
-    TmaMaps tm;
-    memset(&tm, 0, sizeof tm);
-    if (sh.block <= 256) {
-        const int ns = ns_of(type), nc = nc_of(type, a);
-        const bool dbl = a->prec != FE_FP32_MIXED;
-        const uint64_t cs = dbl ? 8 : 4;
-        if (a->coords_layout == FE_LAYOUT_SOA)
-            p.tma_in = encode_planes(tm.x, true, a->coords, uint64_t(a->n_elem), 3 * ns, uint64_t(p.xs) * 8, sh.block) &&
-                       encode_planes(tm.c, dbl, a->coefs, uint64_t(a->n_elem), nc, uint64_t(p.cs) * cs, sh.block);
-        if (o->layout == FE_LAYOUT_SOA)
-            p.tma_out = encode_planes(tm.a, dbl, o->A, uint64_t(a->n_elem), na_out(type, outl), uint64_t(p.os) * cs,
-                                      sh.block) &&
-                        encode_planes(tm.b, dbl, o->b, uint64_t(a->n_elem), ns, uint64_t(p.os) * cs, sh.block);
-    }
 
     CoefFn fn;
     memset(&fn, 0, sizeof fn);
@@ -579,7 +596,7 @@ static bool zero_copy(fe_ctx *ctx, fe_elem_type type, const fe_elem_args *a, con
         if (!dout.A || !dout.b || (o->flags && !dout.flags)) return false;
         dout.memory = FE_MEM_DEVICE;
     }
-    st = launch_set(ctx, type, &da, &dout, ctx->scratch, s);
+    st = launch_set(ctx, type, &da, &dout, ctx->scratch, s, nullptr, nullptr, true);
     if (st == FE_OK) st = cuda_check(ctx, cudaStreamSynchronize(s), "zero-copy integration");
     return true;
 }
