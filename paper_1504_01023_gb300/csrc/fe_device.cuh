@@ -157,6 +157,13 @@ __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.comm
 __device__ __forceinline__ void bulk_wait_read0() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 __device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
+// Programmatic dependent launch. grid_wait: every kernel of launch_set starts with it,
+// before it reads or writes global memory: the kernels before it in the stream are
+// complete then. grid_trigger: the kernel after may be brought onto the SMs (it then
+// waits in grid_wait); called where that is the call's own fix-up.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // Bounded wait on an mbarrier phase. Returns false (and sets the status bit) if
 // the copy has not landed after ~2^22 polls with back-off (seconds); callers
 // then skip their work for this block instead of spinning forever.

@@ -1867,6 +1867,8 @@ __device__ __forceinline__ void elem_tiles(const ElemParams &p, const TmaMaps *t
         fence_mbar_init();
     }
     __syncthreads();
+    grid_wait();
+    if (PREC != FP64) grid_trigger();
     unsigned phase = 0;
     const int B = blockDim.x;
     const int64_t ntiles = (p.n + B - 1) / B;
@@ -1938,6 +1940,8 @@ __device__ __forceinline__ void pair_tiles(const ElemParams &p, const TmaMaps *t
         fence_mbar_init();
     }
     __syncthreads();
+    grid_wait();
+    if (PREC != FP64) grid_trigger();
     unsigned phase = 0;
     const int B = blockDim.x / 2;
     const int64_t ntiles = (p.n + B - 1) / B;
@@ -1987,6 +1991,8 @@ __global__ void __launch_bounds__(256)
         fence_mbar_init();
     }
     __syncthreads();
+    grid_wait();
+    if (PREC != FP64) grid_trigger();
     unsigned phase = 0;
     const int B = (blockDim.x >> 5) * (32 / TPE);
     const int64_t ntiles = (p.n + B - 1) / B;
@@ -2016,6 +2022,8 @@ __global__ void __launch_bounds__(256)
         fence_mbar_init();
     }
     __syncthreads();
+    grid_wait();
+    if (PREC != FP64) grid_trigger();
     unsigned phase = 0;
     const int B = (blockDim.x >> 5) * 2;
     const int64_t ntiles = (p.n + B - 1) / B;
@@ -2119,6 +2127,8 @@ __global__ void __launch_bounds__(ET == TET && PREC != DWORD ? 512 : 256)
     const CT *C = static_cast<const CT *>(p.C);
     CT *Aout = static_cast<CT *>(p.A);
     CT *Bout = static_cast<CT *>(p.B);
+    grid_wait();
+    if (PREC != FP64) grid_trigger();
     const bool n16 = aligned16(p.conn, 0), c16 = aligned16(C, 0);
     const bool o16 = OUTL == AOS && aligned16(Aout, 0) && aligned16(Bout, 0);
     const int64_t stride = int64_t(gridDim.x) * blockDim.x;
@@ -2225,10 +2235,22 @@ __device__ __forceinline__ void fixup_element(const ElemParams &p, int64_t e, co
 // Fix-up kernel of one call: the list written by the main kernel, 32 entries per warp,
 // consecutive groups of 32 to different blocks, so that a short list spreads over
 // the SMs' double pipes (4,000 flagged generic tetrahedra of 400,000: 14.2 us with a
-// block's 256 threads on consecutive entries, all on 16 SMs).
+// block's 256 threads on consecutive entries, all on 16 SMs). The counter is left at
+// zero for the next call, by the last block to have read it (fix_count[1] counts
+// the blocks), which saves that call an operation on its stream.
 template <int ET, int KIND, int PREC, int QUAD, int CPQ, int INL, int OUTL>
 __global__ void __launch_bounds__(256) fixup_kernel(const ElemParams p, const __grid_constant__ CoefFn fn) {
-    const unsigned cnt = *p.fix_count;
+    __shared__ unsigned cnt;
+    grid_wait();
+    if (threadIdx.x == 0) {
+        cnt = *static_cast<volatile unsigned *>(p.fix_count);
+        __threadfence();
+        if (atomicAdd(p.fix_count + 1, 1u) == gridDim.x - 1) {
+            p.fix_count[0] = 0;
+            p.fix_count[1] = 0;
+        }
+    }
+    __syncthreads();
     const unsigned n = cnt < p.fix_cap ? cnt : p.fix_cap;
     const unsigned lane = threadIdx.x & 31u, warps = blockDim.x >> 5;
     for (unsigned g = (threadIdx.x >> 5) * gridDim.x + blockIdx.x; g * 32u < n; g += warps * gridDim.x) {

@@ -27,6 +27,8 @@ __device__ __forceinline__ void plane_elems(const ElemParams &p, const CoefFn *f
     const CT *C = static_cast<const CT *>(p.C);
     CT *Aout = static_cast<CT *>(p.A);
     CT *Bout = static_cast<CT *>(p.B);
+    grid_wait();
+    if (PREC != FP64) grid_trigger();
     const int64_t ntiles = (p.n + blockDim.x - 1) / blockDim.x;
     for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
         if (p.skip_mod > 0 && tile % p.skip_mod == 0) {   // injected fault: no load, no store

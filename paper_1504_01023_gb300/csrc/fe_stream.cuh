@@ -73,6 +73,7 @@ template <int KIND, int QUAD, int CPQ> __device__ __forceinline__ void stream_ti
         fence_mbar_init();
     }
     __syncwarp();
+    grid_wait();
     double *sX = reinterpret_cast<double *>(smem) + warp * 32 * (12 + NC);
     double *sC = sX + 32 * 12;
     const double *C = static_cast<const double *>(p.C);
