@@ -138,6 +138,8 @@ def library_path() -> str:
 def load():
     """Load libfe.so (it must have been built by ``build.build()``)."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is None:
             if not os.path.exists(_build.LIB):
@@ -186,6 +188,14 @@ def make_args(elem_type, coords, coefs, kind, quad, coef_mode, prec, layout, con
     """ElemArgs for torch tensors. SOA: coords (3*NS, E) and coefs (NC, E), unit
     stride along elements, any plane stride. AOS: coords (E, NS, 3), coefs (E, ...).
     INDEXED: coords = nodes (N, 3), conn (E, NS) int32, coefs (E, ...)."""
+    if layout == AOS and coef_mode != COEF_FN_U:
+        # the plain case in one construction (half the time of field by field)
+        assert coords.is_contiguous() and coefs.is_contiguous()
+        assert coords.dtype == torch.float64
+        want = torch.float32 if prec == FP32_MIXED else torch.float64
+        assert coefs.dtype == want, f"coefficients must be {want}"
+        return ElemArgs(coords.shape[0], coords.data_ptr(), AOS, 0, kind, quad, coef_mode, coefs.data_ptr(), AOS, 0,
+                        prec, _mem(coords), None, 0, ordering, None)
     a = ElemArgs()
     a.ordering = ordering
     if coef_mode == COEF_FN_U:
@@ -281,17 +291,13 @@ def alloc_out(elem_type, n, prec, out_layout, device, with_flags=True, pin=False
 
 
 def make_out(A, b, flags, out_layout, packed=False):
-    o = Out()
-    o.packed = 1 if packed else 0
-    o.A, o.b = A.data_ptr(), b.data_ptr()
-    o.layout = out_layout
+    stride = 0
     if out_layout == SOA:
         n = A.shape[1]
         assert n <= 1 or (A.stride(0) == b.stride(0) and A.stride(1) == 1 and b.stride(1) == 1)
-        o.stride = A.stride(0) if n > 1 else 0
-    o.flags = flags.data_ptr() if flags is not None else None
-    o.memory = _mem(A)
-    return o
+        stride = A.stride(0) if n > 1 else 0
+    return Out(A.data_ptr(), b.data_ptr(), out_layout, stride, flags.data_ptr() if flags is not None else None, _mem(A),
+               1 if packed else 0)
 
 
 # Largest n_elem fe_integrate_tet_noalloc accepts (its static scratch holds one
@@ -336,6 +342,11 @@ def context_settings(autotune=None, tuning_cache=None, environ=None):
     return bool(autotune), tuning_cache
 
 
+# the handle of a device's current stream, without the Stream object around it
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None) or (
+    lambda device: torch.cuda.current_stream(device).cuda_stream)
+
+
 class Context:
     """One library context on one CUDA device."""
 
@@ -375,7 +386,7 @@ class Context:
         if stream is not None:
             return ctypes.c_void_p(stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream))
         if on_device:
-            return ctypes.c_void_p(torch.cuda.current_stream(self.device).cuda_stream)
+            return ctypes.c_void_p(_raw_stream(self.device))
         return ctypes.c_void_p(0)
 
     def integrate(self, elem_type, coords, coefs, kind, quad, coef_mode=PER_ELEMENT, prec=FP32_MIXED, layout=SOA,

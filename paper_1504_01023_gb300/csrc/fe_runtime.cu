@@ -9,6 +9,7 @@
 #include <fstream>
 #include <mutex>
 #include <sstream>
+#include <tuple>
 
 #include <cudaTypedefs.h>
 
@@ -210,13 +211,33 @@ fe_status set_smem_attr(fe_ctx *ctx, const void *k, int64_t smem) {
     return e;
 }
 
+// Blocks of a launch resident on one SM; a property of kernel and shape, looked up
+// once for each (the runtime's answer takes about a microsecond).
+static int resident_blocks(int device, const void *k, int threads, int64_t smem) {
+    static std::mutex mu;
+    static std::map<std::tuple<int, const void *, int, int64_t>, int> known;
+    std::lock_guard<std::mutex> lk(mu);
+    int &n = known[{device, k, threads, smem}];
+    if (n == 0) {
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, threads, size_t(smem));
+        n = std::max(n, 1);
+    }
+    return n;
+}
+
+// "t0k1p1q1c0i1o1r0n8": type, kind, precision, rule, coefficient mode, layouts, loop
+// ordering (one digit each) and size class floor(log4 n). Formatted by hand: two
+// string streams per call took 2 of its 6 us on the host.
 static std::string shape_key(fe_elem_type type, const fe_elem_args *a, const fe_out *o) {
     int bucket = 0;
-    for (int64_t n = a->n_elem; n > 1; n >>= 2) ++bucket;  // size class: floor(log4 n)
-    std::ostringstream k;
-    k << "t" << type << "k" << a->kind << "p" << a->prec << "q" << a->quad << "c" << a->coef_mode << "i"
-      << a->coords_layout << "o" << out_mode(o) << "r" << a->ordering << "n" << bucket;
-    return k.str();
+    for (int64_t n = a->n_elem; n > 1; n >>= 2) ++bucket;
+    char k[24] = "t0k0p0q0c0i0o0r0n";
+    const int v[8] = {type, a->kind, a->prec, a->quad, a->coef_mode, a->coords_layout, out_mode(o), a->ordering};
+    for (int i = 0; i < 8; ++i) k[2 * i + 1] = char('0' + v[i]);
+    int len = 17;
+    if (bucket >= 10) k[len++] = char('0' + bucket / 10);
+    k[len++] = char('0' + bucket % 10);
+    return std::string(k, size_t(len));
 }
 
 Shape default_shape(fe_elem_type type) { return Shape{type == FE_TET ? 256 : 128, 0}; }
@@ -376,9 +397,7 @@ fe_status launch_set(fe_ctx *ctx, fe_elem_type type, const fe_elem_args *a, cons
     const int64_t ntiles = (a->n_elem + sh.block - 1) / sh.block;
     int64_t grid = ntiles;
     if (sh.persistent) {
-        int per_sm = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, size_t(smem));
-        grid = std::min<int64_t>(ntiles, int64_t(std::max(per_sm, 1)) * ctx->sms);
+        grid = std::min<int64_t>(ntiles, int64_t(resident_blocks(ctx->device, k, threads, smem)) * ctx->sms);
     }
     grid = std::min<int64_t>(grid, 0x7FFFFFFF);
 
