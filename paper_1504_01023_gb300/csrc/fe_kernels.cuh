@@ -895,14 +895,22 @@ template <int KIND, int CPQ> struct ElemMath<PRISM, KIND, FP64, Q_PRISM6, CPQ> {
         P.template sums<KIND>();
         P.template align<KIND>(min(P.lza, __shfl_xor_sync(mask, P.lza, 1)), min(P.lzb, __shfl_xor_sync(mask, P.lzb, 1)));
 #pragma unroll
-        for (int i = 0; i < 9; ++i) {
-            long long X, Y, U, V;
-            P.blocks(part, i, X, Y, U, V);
-            const long long p = (part ? U : X) + __shfl_xor_sync(mask, part ? X : U, 1);
-            const long long q = (part ? V : Y) + __shfl_xor_sync(mask, part ? Y : V, 1);
-            Ah[i] = P.out_a(p + q);
-            Ah[9 + i] = P.out_a(p - q);
-        }
+        for (int k = 0; k < 3; ++k)
+#pragma unroll
+            for (int kk = KIND == POISSON ? k : 0; kk < 3; ++kk) {
+                const int i = 3 * k + kk, it = 3 * kk + k;
+                long long X, Y, U, V;
+                P.blocks(part, i, X, Y, U, V);
+                const long long p = (part ? U : X) + __shfl_xor_sync(mask, part ? X : U, 1);
+                const long long q = (part ? V : Y) + __shfl_xor_sync(mask, part ? Y : V, 1);
+                Ah[i] = P.out_a(p + q);
+                Ah[9 + i] = P.out_a(p - q);
+                if (KIND == POISSON && k != kk) {
+                    // symmetric: the diagonal blocks each, the off-diagonal ones to one another
+                    Ah[it] = part ? Ah[9 + i] : Ah[i];
+                    Ah[9 + it] = part ? Ah[i] : Ah[9 + i];
+                }
+            }
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
             long long X, Y;
@@ -1968,7 +1976,8 @@ __global__ void __launch_bounds__(256)
 // in the double form, which the double pipe bounded at 0.89 of its rate). 400,000
 // prisms with per-point coefficients: 0.376 -> 1.29 Gelem/s (128 registers 1.09, 168
 // 1.25, 200 1.29, 255 1.28), per-element 1.36 (168 registers 1.29, 255 1.36),
-// Laplace 1.04 -> 2.80 (96 registers 2.76, 128 2.80, 168 2.64).
+// Laplace 1.04 -> 2.80 (96 registers 2.76, 128 2.80, 168 2.64), 2.95 with the six upper
+// entries of each symmetric block only (500,000 prisms 176 -> 168 us).
 template <int KIND, int CPQ>
 __global__ void __launch_bounds__(256) __maxnreg__(KIND == POISSON ? 128 : (CPQ ? 200 : 255))
     pair_kernel_f64(const ElemParams p, const __grid_constant__ TmaMaps tm, const __grid_constant__ CoefFn fn) {
