@@ -69,6 +69,7 @@ struct PrismFx {
     int64_t *v;
     FxRange gb, g3, gv;
     int64_t SV[9], SW[2][6];   // the value row's part of SF, and of SP and SQ
+    int64_t s4[4], p2[2][3], q2[2][3];
 
     FE_HD static void negate(const Fx2 a[3], Fx2 n[3]) {   // a's low limbs are above -2^31
 #pragma unroll
@@ -465,46 +466,43 @@ struct PrismFx {
     // The level's sums over its points
     template <int KIND> FE_HD void sums() {
         ok = ok && gb.bits() < kGammaHi && g3.bits() < kGamma3Hi && gv.bits() < kValueHi;
-        // sums with the points' weights
-        int64_t wa[3], wb[3];
+        // sums with the points' weights; SF, SP and SQ are expanded from s4, p2 and q2 in
+        // align (4 and 6 + 6 values across the exchange between the two threads instead of
+        // 27: the per-point generic kernel fits 168 registers, 300,000 prisms 242 -> 224 us)
         if (KIND == 0) {
-            S.SF[4] = S4[0];
-            S.SF[5] = S.SF[7] = S4[1];
-            S.SF[8] = S4[2];
-            weighted(G13, wa);
-            weighted(G23, wb);
-            pi(wa, wb, S.SP, false);
-            pi(wa, wb, S.SQ, true);
+            s4[0] = S4[0];
+            s4[1] = s4[2] = S4[1];
+            s4[3] = S4[2];
+            weighted(G13, p2[0]);
+            weighted(G23, p2[1]);
             weighted2(G33, S.SG);
             weighted(d0, S.BU);
             S.BR[0] = S.BR[1] = S.BR[2] = 0;
         } else {
-            int64_t w2[6], e1[3], e2[3];
+            int64_t w2[6], e1[3], e2[3], f1[3], f2[3];
             weighted2(at(0), w2);
             weighted(at(1), e1);
             weighted(at(2), e2);
-            weighted(at(4), wa);
-            weighted(at(5), wb);
+            weighted(at(4), f1);
+            weighted(at(5), f2);
 #pragma unroll
             for (int k = 0; k < 3; ++k)
 #pragma unroll
                 for (int kk = 0; kk < 3; ++kk) {
                     const int64_t de = kk == 0 ? -(e1[k] + e2[k]) : (kk == 1 ? e1[k] : e2[k]);
-                    const int64_t df = k == 0 ? -(wa[kk] + wb[kk]) : (k == 1 ? wa[kk] : wb[kk]);
+                    const int64_t df = k == 0 ? -(f1[kk] + f2[kk]) : (k == 1 ? f1[kk] : f2[kk]);
                     SV[3 * k + kk] = w2[k == kk ? k : k + kk + 2] + de + df;
                 }
             weighted2(at(3), SW[0]);
             weighted2(at(6), SW[1]);
-            S.SF[4] = at(7).sum();
-            S.SF[5] = at(8).sum();
-            S.SF[7] = at(10).sum();
-            S.SF[8] = at(11).sum();
-            weighted(at(9), wa);
-            weighted(at(12), wb);
-            pi(wa, wb, S.SP, false);
-            weighted(at(13), wa);
-            weighted(at(14), wb);
-            pi(wa, wb, S.SQ, true);
+            s4[0] = at(7).sum();
+            s4[1] = at(8).sum();
+            s4[2] = at(10).sum();
+            s4[3] = at(11).sum();
+            weighted(at(9), p2[0]);
+            weighted(at(12), p2[1]);
+            weighted(at(13), q2[0]);
+            weighted(at(14), q2[1]);
             weighted2(at(15), S.SG);
             weighted(at(16), S.BU);
             const int64_t l1 = at(17).sum(), l2 = at(18).sum();
@@ -513,40 +511,46 @@ struct PrismFx {
             S.BU[2] += l2;
             weighted(at(19), S.BR);
         }
-        S.SF[3] = -(S.SF[4] + S.SF[5]);
-        S.SF[6] = -(S.SF[7] + S.SF[8]);
-        S.SF[1] = -(S.SF[4] + S.SF[7]);
-        S.SF[2] = -(S.SF[5] + S.SF[8]);
-        S.SF[0] = (S.SF[4] + S.SF[5]) + (S.SF[7] + S.SF[8]);
         // leading zeros in units of SF and of BU: to agree on the units of the sums over
         // both levels
         dV = sV - s12;
         dW = dz + sV - s12;
         dP = dz + s3 - s12;
-        dQ = KIND == 0 ? dP : dz;   // Laplace: SQ is SP transposed
+        dQ = dz;
         dG = 2 * dz + s3 - s12;
         uint32_t bf = 0, bp = 0, bq = 0, bg = 0, bu = 0, br = 0, bv = 0, bw = 0;
+        {
+            // (as they come out of align)
+            int64_t w[9];
+            expand4(s4, w);
 #pragma unroll
-        for (int k = 0; k < 9; ++k) {
-            bf |= fx_hi_bits(S.SF[k]);
-            bp |= fx_hi_bits(S.SP[k]);
-            bq |= fx_hi_bits(S.SQ[k]);
-            if (KIND == 1) bv |= fx_hi_bits(SV[k]);
+            for (int k = 0; k < 9; ++k) bf |= fx_hi_bits(w[k]);
+            pi(p2[0], p2[1], w, false);
+#pragma unroll
+            for (int k = 0; k < 9; ++k) bp |= fx_hi_bits(w[k]);
+            if (KIND == 1) {
+                pi(q2[0], q2[1], w, true);
+#pragma unroll
+                for (int k = 0; k < 9; ++k) bq |= fx_hi_bits(w[k]);
+            }
         }
-        if (KIND == 1)
+        if (KIND == 1) {
+#pragma unroll
+            for (int k = 0; k < 9; ++k) bv |= fx_hi_bits(SV[k]);
 #pragma unroll
             for (int k = 0; k < 6; ++k) bw |= fx_hi_bits(SW[0][k]) | fx_hi_bits(SW[1][k]);
+        }
 #pragma unroll
         for (int k = 0; k < 6; ++k) bg |= fx_hi_bits(S.SG[k]);
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
             bu |= fx_hi_bits(S.BU[k]);
-            br |= fx_hi_bits(S.BR[k]);
+            if (KIND == 1) br |= fx_hi_bits(S.BR[k]);
         }
         // (minima of the leading zeros: nvcc 13.0 compiled the maxima of their negatives to
         // the maximum of the magnitudes)
-        lza = fx_mini(fx_mini(fx_clz(bf), fx_clz(bp) + dP), fx_mini(fx_clz(bq) + dQ, fx_clz(bg) + dG));
-        if (KIND == 1) lza = fx_mini(lza, fx_mini(fx_clz(bv) + dV, fx_clz(bw) + dW));
+        lza = fx_mini(fx_mini(fx_clz(bf), fx_clz(bp) + dP), fx_clz(bg) + dG);
+        if (KIND == 1) lza = fx_mini(fx_mini(lza, fx_clz(bq) + dQ), fx_mini(fx_clz(bv) + dV, fx_clz(bw) + dW));
         lzb = fx_mini(fx_clz(bu), fx_clz(br) + dz);
     }
     // Brings the level's sums to common units from the smaller leading zeros of the two
@@ -560,12 +564,19 @@ struct PrismFx {
         const int sa = za - 6, sb = zb - 5;
         xg = xgamma<KIND>() - s12 - sa;
         xl = xload() - sb;
+        int64_t f[4];
 #pragma unroll
-        for (int k = 0; k < 9; ++k) {
-            S.SF[k] = shift(S.SF[k], sa);
-            S.SP[k] = shift(S.SP[k], sa - dP);
-            S.SQ[k] = shift(S.SQ[k], sa - dQ);
-            if (KIND == 1) S.SF[k] += shift(SV[k], sa - dV);
+        for (int k = 0; k < 4; ++k) f[k] = KIND == 0 && k == 2 ? f[1] : shift(s4[k], sa);
+        expand4(f, S.SF);
+        shift3(p2, sa - dP);
+        pi(p2[0], p2[1], S.SP, false);
+        if (KIND == 0) {
+            pi(p2[0], p2[1], S.SQ, true);
+        } else {
+            shift3(q2, sa - dQ);
+            pi(q2[0], q2[1], S.SQ, true);
+#pragma unroll
+            for (int k = 0; k < 9; ++k) S.SF[k] += shift(SV[k], sa - dV);
         }
         if (KIND == 1) {
             int64_t p[2][6];
@@ -587,7 +598,26 @@ struct PrismFx {
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
             S.BU[k] = shift(S.BU[k], sb);
-            S.BR[k] = shift(S.BR[k], sb - dz);
+            if (KIND == 1) S.BR[k] = shift(S.BR[k], sb - dz);
+        }
+    }
+    // D s D^T for the 2 x 2 matrix s (row-major), D = [-1 -1; 1 0; 0 1]
+    FE_HD static void expand4(const int64_t s[4], int64_t w[9]) {
+        w[4] = s[0];
+        w[5] = s[1];
+        w[7] = s[2];
+        w[8] = s[3];
+        w[3] = -(s[0] + s[1]);
+        w[6] = -(s[2] + s[3]);
+        w[1] = -(s[0] + s[2]);
+        w[2] = -(s[1] + s[3]);
+        w[0] = (s[0] + s[1]) + (s[2] + s[3]);
+    }
+    FE_HD static void shift3(int64_t w[2][3], int n) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            w[0][k] = shift(w[0][k], n);
+            w[1][k] = shift(w[1][k], n);
         }
     }
     // This level's share of the four blocks (see the FP64 form's pair_blocks), doubled:

@@ -1974,12 +1974,13 @@ __global__ void __launch_bounds__(256)
 // its chains at 8 to 16 warps per SM (6,500 instructions per thread, half of them
 // 32-bit integer operations; 51 double instructions against about 1,500 per element
 // in the double form, which the double pipe bounded at 0.89 of its rate). 400,000
-// prisms with per-point coefficients: 0.376 -> 1.29 Gelem/s (128 registers 1.09, 168
-// 1.25, 200 1.29, 255 1.28), per-element 1.36 (168 registers 1.29, 255 1.36),
-// Laplace 1.04 -> 2.80 (96 registers 2.76, 128 2.80, 168 2.64), 2.95 with the six upper
-// entries of each symmetric block only (500,000 prisms 176 -> 168 us).
+// prisms with per-point coefficients: 0.376 -> 1.32 Gelem/s (128 registers 1.16, 168
+// 1.32, 200 1.27, 255 1.27; 300,000 in a call 819 -> 224 us), per-element 1.36 (168
+// registers 1.29, 255 1.36), Laplace 1.04 -> 2.87 (96 registers 2.84, 128 2.87, 168 2.71;
+// 500,000 in a call 493 -> 166 us, 176 before only the six upper entries of each
+// symmetric block were formed).
 template <int KIND, int CPQ>
-__global__ void __launch_bounds__(256) __maxnreg__(KIND == POISSON ? 128 : (CPQ ? 200 : 255))
+__global__ void __launch_bounds__(256) __maxnreg__(KIND == POISSON ? 128 : (CPQ ? 168 : 255))
     pair_kernel_f64(const ElemParams p, const __grid_constant__ TmaMaps tm, const __grid_constant__ CoefFn fn) {
     pair_tiles<KIND, FP64, CPQ>(p, &tm, &fn);
 }
