@@ -3,6 +3,8 @@ warp's 16 elements and a block's tile, several tiles per block, records off thei
 16-byte boundaries, and warps that mix ordinary elements with elements outside the
 fixed-point windows, against the oracle (1e-12 per element, the FP64 form's
 tolerance) and, for those elements, against the one-thread double form."""
+import time
+
 import numpy as np
 import pytest
 import torch
@@ -84,3 +86,24 @@ def test_elements_outside_the_windows(ctx, kind, cpq):
     scale = np.abs(A1[keep]).reshape(keep.sum(), -1).max(1)[:, None, None]
     assert oracle.rel_frobenius(A[keep] / scale, A1[keep] / scale).max() <= 1e-12
     assert np.isfinite(A).all() and np.isfinite(b).all()
+
+
+@pytest.mark.parametrize("kind,cpq", CASES)
+def test_served_requests(ctx, kind, cpq):
+    """Served FP64 prisms (two threads each) against the oracle."""
+    for n in (1, 33, 1003):
+        mesh, c = _inputs(n, kind, cpq)
+        Ao, bo, _ = oracle.integrate(oracle.PRISM, kind, oracle.Q_PRISM6, mesh, c, coef_per_q=bool(cpq), n_threads=8)
+        mid = ctx.mesh_register(api.PRISM, torch.from_numpy(mesh).cuda(), api.AOS)
+        C = torch.from_numpy(c).cuda()
+        tk = ctx.serve_submit(mid, kind, api.QUAD_PRISM6, api.PER_QPOINT if cpq else api.PER_ELEMENT, C, prec=api.FP64)
+        t0 = time.time()
+        while (r := ctx.serve_poll(tk)) is None:
+            assert time.time() - t0 < 30.0, "request did not finish"
+            time.sleep(0.0005)
+        A, b, f = ctx.serve_result_tensors(tk, r)
+        assert oracle.rel_frobenius(A.cpu().numpy(), Ao).max() <= TOL[api.FP64]
+        assert oracle.rel_frobenius(b.cpu().numpy(), bo).max() <= TOL[api.FP64]
+        assert (f.cpu().numpy() == 0).all()
+        ctx.serve_release(tk)
+        ctx.mesh_release(mid)
