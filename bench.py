@@ -243,7 +243,8 @@ def paper_context():
 
 # GB300 HBM3e nominal bandwidth (GB/s), reported beside the measured copy ceiling
 NOMINAL_HBM_GBS = 7900.0
-# FP64 pipe: 2 instructions per clock per SM (the nominal 1.25 TFLOP/s of FMAs);
+# FP64 pipe: 2 instructions per clock per SM (the nominal 1.25 TFLOP/s of FMAs; the
+# block fixed-point kernels leave it 34 instructions per generic tetrahedron);
 # instruction issue: one warp instruction per clock per SM sub-partition (4 per SM)
 FP64_PIPE_PER_CLK_SM = 2
 ISSUE_PER_CLK_SM = 4 * 32
@@ -484,7 +485,7 @@ def run_native(args):
         wl_name = {"fp64": WORKLOAD, "mixed": MIXED_WORKLOAD}.get(args.form, MESH + ", double-word form")
         if lap:
             wl_name = MESH.split(", TET4")[0] + ", Laplace operator, TET1, d^0 = 1, " + args.form + " form"
-        kname = {"fp64": "elem_kernel_f64t", "dw": "elem_kernel_dwt"}.get(args.form, "elem_kernel")
+        kname = {"fp64": "stream_kernel_f64t", "dw": "elem_kernel_dwt"}.get(args.form, "elem_kernel")
         kernel_name = (f"{kname}<TET,{'POISSON' if lap else 'GENERIC'},{PREC_TAG[args.form]},"
                        f"{'TET1' if lap else 'TET4'},per-element,AOS,AOS>")
         tag = f"tet_{'poisson_tet1' if lap else 'generic'}_{args.form}_aos"
@@ -496,7 +497,8 @@ def run_native(args):
         kw = dict(kind=api.POISSON if lap else api.GENERIC, quad=api.QUAD_PRISM6, coef_mode=api.PER_QPOINT,
                   prec=prec, layout=api.AOS, out_layout=api.AOS)
         wl_name = PRISM_WORKLOAD
-        kernel_name = f"elem_kernel<PRISM,{'POISSON' if lap else 'GENERIC'},{PREC_TAG[args.form]},PRISM6,per-point,AOS,AOS>"
+        kernel_name = (f"{'pair_kernel_f64' if args.form == 'fp64' else 'elem_kernel'}<PRISM,"
+                       f"{'POISSON' if lap else 'GENERIC'},{PREC_TAG[args.form]},PRISM6,per-point,AOS,AOS>")
         tag = f"prism_{'poisson' if lap else 'generic'}_{args.form}_aos"
     n = len(mesh)
     X = torch.from_numpy(np.ascontiguousarray(mesh)).to(dev)                       # [E,NS,3] f64
@@ -551,12 +553,11 @@ def run_native(args):
     if args.form == "mixed":
         roofline = hbm
     else:
-        # the double-precision forms are bound by an instruction rate, not by HBM:
-        # the FP64 pipe (plain FP64) or instruction issue (double-word); the HBM
-        # figures stay beside it
-        pipe = (FP64_PIPE_PER_CLK_SM, "FP64-pipe", "fp64_pipe_inst_per_elem") if args.form == "fp64" else \
-            (ISSUE_PER_CLK_SM, "thread", "inst_per_elem")
-        roofline = pipe_roofline(melem_k, ncu_record(tag, pipe[2]), sms, sm_mhz, pipe[0], pipe[1], tag)
+        # the double-precision forms (plain FP64 in block fixed point, double-word in
+        # float pairs) are bound by instruction issue before HBM; the HBM figures stay
+        # beside it
+        roofline = pipe_roofline(melem_k, ncu_record(tag, "inst_per_elem"), sms, sm_mhz, ISSUE_PER_CLK_SM, "thread",
+                                 tag)
         roofline.update(kernel=kernel_name, kernel_ms=k_ms, traffic=hbm["traffic"],
                         hbm={k: hbm[k] for k in ("achieved", "peak", "unit", "frac", "peak_kind",
                                                  "algorithmic_bytes_per_launch", "frac_of_nominal",
@@ -952,8 +953,7 @@ def coef_function_form(ctx, dev, api, args):
 
 def _fp64_run(ctx, dev, api, X, C, et, kind, quad, prec, args, cm=None, rates=None, tag=None):
     """Tuned shape, then the average kernel time (profiling events) of repeated
-    calls; with `tag`, the instruction-rate roofline of the form (FP64 pipe for
-    plain FP64, instruction issue for double-word) from that ncu record."""
+    calls; with `tag`, the instruction-issue roofline from that ncu record."""
     import torch
     n = X.shape[0]
     cm = api.PER_ELEMENT if cm is None else cm
@@ -974,12 +974,8 @@ def _fp64_run(ctx, dev, api, X, C, et, kind, quad, prec, args, cm=None, rates=No
            "achieved_gbs": gbs, "hbm_frac": gbs / peak, "peak_source": src, "flagged_to_fp64": flagged,
            "launch_shape": shape_dict(shape)}
     if tag is not None and rates is not None:
-        if prec == api.FP64:
-            res["fp64_pipe"] = pipe_roofline(res["value"], ncu_record(tag, "fp64_pipe_inst_per_elem"), rates["sms"],
-                                             rates["sm_mhz"], FP64_PIPE_PER_CLK_SM, "FP64-pipe", tag)
-        else:
-            res["issue"] = pipe_roofline(res["value"], ncu_record(tag, "inst_per_elem"), rates["sms"],
-                                         rates["sm_mhz"], ISSUE_PER_CLK_SM, "thread", tag)
+        res["issue"] = pipe_roofline(res["value"], ncu_record(tag, "inst_per_elem"), rates["sms"], rates["sm_mhz"],
+                                     ISSUE_PER_CLK_SM, "thread", tag)
     return res
 
 
@@ -1010,7 +1006,7 @@ def double_forms(ctx, dev, api, X, coefs, args, rates):
              "roofline": dw_gen.get("issue"), "generic_tet4": dw_gen, "poisson_tet1": dw_lap}
     fp64 = {"workload": wl + "; Laplace operator, TET1, d^0 = 1 (the 48,000-element Poisson workload scaled)",
             "value": nat_lap["value"], "unit": "Melem/s", "hbm_frac": nat_lap["hbm_frac"], "dtype": "f64",
-            "roofline": nat_lap.get("fp64_pipe"), "poisson_tet1": nat_lap}
+            "roofline": nat_lap.get("issue"), "poisson_tet1": nat_lap}
     return dword, fp64
 
 

@@ -62,7 +62,10 @@ typedef enum fe_elem_type { FE_TET = 0, FE_PRISM = 1 } fe_elem_type;
    d^0 per integration point; "conv-diff" (here FE_GENERIC) = all 16 c and 4 d. */
 typedef enum fe_problem { FE_POISSON = 0, FE_GENERIC = 1 } fe_problem;
 
-/* FE_FP64: all arithmetic in double, inputs and outputs double.
+/* FE_FP64: inputs and outputs double, double accuracy: on the GPU tetrahedra, and
+   prisms with two threads per element, compute in 61-bit integers with shared
+   exponents (error against exact results no larger than double arithmetic's) and
+   in double whatever leaves that range; the rest in double throughout.
    FE_FP32_MIXED: coordinates stay double in memory; edge vectors are formed
    exactly enough in single precision, the coefficient and shape-derivative
    arithmetic and accumulation run in float, coefficients and outputs are float.

@@ -2,9 +2,10 @@
 // even), computed with 32-bit integer instructions.
 //
 // This GPU issues double-precision instructions at 2 per clock per SM and
-// integer instructions at 64 per clock per SM per pipe. The plain FP64 kernels
-// are bound by the double pipe while the integer pipes idle, so they run a part
-// of their double multiplications and additions here instead. These are the
+// integer instructions at 64 per clock per SM per pipe. The FP64 arithmetic in
+// doubles (per-point tetrahedra, one-thread prisms and what leaves the windows of
+// the block fixed point) is bound by the double pipe while the integer pipes idle,
+// so it runs a part of its multiplications and additions here instead. These are the
 // same IEEE operations, not approximations: for normal operands and a normal
 // result the value returned is the correctly rounded product or sum, bit for
 // bit what the double-precision instruction returns; so is the signed zero of a

@@ -173,8 +173,8 @@ template <int KIND, int QUAD, int CPQ> __device__ __forceinline__ void stream_ti
     }
 }
 
-// Registers: generic 128 (3M TET4: 72 registers 9.20, 80 9.95, 96 10.31, 104 10.40,
-// 128 10.74 Gelem/s: fewer spills and more independent chains outweigh the warps),
+// Registers: generic 128 (3M TET4: 104 registers 10.61, 128 10.85, 144 10.27, 168 9.89
+// Gelem/s: above, fewer warps; below, spills and fewer independent chains),
 // Laplace 64 (TET1: 48 18.2, 56 19.05, 64 19.1, 80 18.7).
 template <int KIND, int QUAD, int CPQ>
 __global__ void __launch_bounds__(512) __maxnreg__(KIND == POISSON ? 64 : 128)
