@@ -27,6 +27,9 @@ template <int ET, int KIND, int PREC, int QUAD, int CPQ, int INL, int OUTL> cons
 #define FE_PLANE_CASE(ET, PREC, QUAD, KD, CP, IL, OL)                                 \
     if (kind == KD && prec == PREC && quad == QUAD && cpq == CP && outl == OL)       \
         return reinterpret_cast<const void *>(&fe::plane_kernel<ET, KD, PREC, QUAD, CP, OL>);
+#define FE_PLANE_PAIR_CASE(ET, PREC, QUAD, KD, CP, IL, OL)                            \
+    if (kind == KD && prec == PREC && quad == QUAD && cpq == CP && outl == OL)       \
+        return reinterpret_cast<const void *>(&fe::plane_pair_kernel<KD, CP, OL>);
 #define FE_FIX_CASE(ET, PREC, QUAD, KD, CP, IL, OL)                                   \
     if (kind == KD && cpq == CP && inl == IL && outl == OL)                          \
         return reinterpret_cast<const void *>(&fe::fixup_kernel<ET, KD, PREC, QUAD, CP, IL, OL>);

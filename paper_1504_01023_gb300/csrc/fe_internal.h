@@ -91,17 +91,23 @@ const void *kernel_group_prism(int kind, int prec, int cpq);
 // Plane-major in and out, straight from and to global memory (fe_plane.cuh).
 const void *kernel_plane_tet(int kind, int prec, int quad, int cpq, int outl);
 const void *kernel_plane_prism(int kind, int prec, int quad, int cpq, int outl);
+// Dynamic shared memory of those kernels: 60 values per thread for FP64 generic
+// prisms (plane_pair_kernel).
+constexpr int64_t plane_smem(int type, int kind, int prec, int threads) {
+    return type == PRISM && prec == FP64 && kind == GENERIC ? int64_t(threads) * 480 : 0;
+}
 // Forms whose plane-major sets always take those kernels; the others take tiles
 // moved by tensor copies where the planes' alignment allows these. Measured on
 // aligned planes, tensor copies / straight, us: 3M FP64 tets generic 752 (of them
 // 350 the double form) / 304 and Laplace 277 / 155; 6M mixed tets generic 253 / 246,
 // but Laplace 171 / 179; 3M double-word tets generic 350 / 380, Laplace 157 / 162; 1M
 // mixed prisms Laplace 72 / 64, generic per element 130 / 120, but per point 147 / 235
-// (120 coefficient planes). Without alignment the tile kernel copies value by value:
+// (120 coefficient planes); 300k FP64 prisms (one thread in doubles / two in fixed
+// point) generic per point 845 / 248, Laplace 311 / 116. Without alignment the tile kernel copies value by value:
 // 400k mixed generic tets 71 / 24, 1M mixed generic prisms per point 1,925 / 235.
 constexpr bool plane_always(int type, int kind, int prec, int cpq) {
     return type == TET ? prec == FP64 || (prec == MIXED && kind == GENERIC)
-                       : prec == MIXED && (kind == POISSON || cpq == 0);
+                       : prec == FP64 || (prec == MIXED && (kind == POISSON || cpq == 0));
 }
 
 // Fix-up kernels (flagged elements of the mixed and double-word forms, redone

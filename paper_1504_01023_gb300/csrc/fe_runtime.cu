@@ -387,7 +387,8 @@ fe_status launch_set(fe_ctx *ctx, fe_elem_type type, const fe_elem_args *a, cons
                     : !stream && sh.tpe == 1 && stream_ok(type, a, outl)     ? kernel_tet_fp64_tile(a->kind, a->quad, cpq_of(a))
                                                                              : main_kernel(type, a, outl, sh.tpe);
     if (!k) return set_error(ctx, FE_ERR_UNSUPPORTED, "no kernel for this combination");
-    const int64_t smem = planes ? 0 : smem_bytes(type, a, outl, sh.block, sh.tpe, stream);
+    const int64_t smem = planes ? plane_smem(type, a->kind, a->prec, threads)
+                                : smem_bytes(type, a, outl, sh.block, sh.tpe, stream);
     if (smem + kStaticSmem > ctx->max_smem_optin)
         return set_error(ctx, FE_ERR_UNSUPPORTED, "shared memory of this launch shape too large");
     {

@@ -107,3 +107,46 @@ def test_served_requests(ctx, kind, cpq):
         assert (f.cpu().numpy() == 0).all()
         ctx.serve_release(tk)
         ctx.mesh_release(mid)
+
+
+@pytest.mark.parametrize("kind,cpq", CASES)
+@pytest.mark.parametrize("n,shape", [(1, (32, 0)), (15, (32, 0)), (17, (64, 1)), (33, (32, 1)), (1003, (128, 0)),
+                                     (2500, (96, 1)), (4999, (32, 1))])
+def test_plane_major(ctx, kind, cpq, n, shape):
+    """Plane-major sets: the bits of the element-contiguous pair kernel, and for
+    elements outside the windows (double arithmetic, contracted as each kernel's
+    compilation has it) its values within the FP64 tolerance; planes off their 16-byte boundaries, a pitch longer
+    than the set, and the Laplace kind's packed output."""
+    mesh, c = _inputs(n, kind, cpq)
+    inside = np.ones(n, dtype=bool)
+    if n > 1000:
+        mesh[3::11] *= 2.0 ** 120
+        mesh[5::13, 3:] = mesh[5::13, :3]
+        inside[3::11] = inside[5::13] = False
+    A, b, f = _run(ctx, mesh, c, kind, cpq, (32, 0), 2)
+    kw = dict(kind=kind, quad=api.QUAD_PRISM6, coef_mode=api.PER_QPOINT if cpq else api.PER_ELEMENT, prec=api.FP64,
+              layout=api.SOA, out_layout=api.SOA)
+
+    def planes(v, off):
+        t = torch.empty(v.size + off, dtype=torch.float64, device="cuda")[off:].view(-1, n)
+        return t.copy_(torch.from_numpy(np.ascontiguousarray(v.reshape(n, -1).T)))
+
+    for off in (0, 1):
+        X, C = planes(mesh, off), planes(c, off)
+        for packed in ((False, True) if kind == api.POISSON else (False,)):
+            na = 21 if packed else 36
+            buf = [torch.full((n * k + 4,), 77.0, dtype=torch.float64, device="cuda") for k in (na, 6)]
+            out = (buf[0][:n * na].view(na, n), buf[1][:n * 6].view(6, n),
+                   torch.full((n,), 99, dtype=torch.uint8, device="cuda"))
+            ctx.set_shape(shape[0], shape[1], api.PRISM, X, C, out=out, packed=packed, **kw)
+            ctx.integrate(api.PRISM, X, C, out=out, packed=packed, **kw)
+            ctx.sync()
+            ref = A.reshape(n, 36)
+            if packed:
+                ref = A[:, np.triu_indices(6)[0], np.triu_indices(6)[1]]
+            for got, want in ((out[0].cpu().numpy().T, ref), (out[1].cpu().numpy().T, b)):
+                assert np.array_equal(got[inside], want[inside])
+                err = np.linalg.norm(got - want, axis=1)
+                assert (err <= TOL[api.FP64] * np.linalg.norm(want, axis=1)).all()
+            assert np.array_equal(out[2].cpu().numpy(), f)
+            assert (buf[0][n * na:] == 77).all() and (buf[1][n * 6:] == 77).all()
