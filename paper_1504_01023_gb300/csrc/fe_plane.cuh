@@ -80,7 +80,8 @@ __global__ void __launch_bounds__(ET == TET && PREC != DWORD ? 512 : 256)
 // of A^e and b^e. Against the tensor-copied tiles of one thread in doubles, us:
 // 300,000 per point 845 / 248, per element 860 / 226, Laplace 311 / 116; 20,000 per
 // point 89 / 33, Laplace 35 / 19; 200,000 per point in pinned host memory 1,228 /
-// 1,120. Generic kind: 60 values of dynamic shared memory per thread, its point coefficients first (read several times), then PrismFx's own.
+// 1,120. Generic kind: 60 values of dynamic shared memory per thread, its point
+// coefficients first (read several times), then PrismFx's own.
 // Tiles of blockDim elements in two passes, so that a launch shape means the same
 // elements per block as in the other plane-major kernels.
 template <int KIND, int CPQ, int OUTL>
