@@ -64,8 +64,9 @@ typedef enum fe_problem { FE_POISSON = 0, FE_GENERIC = 1 } fe_problem;
 
 /* FE_FP64: inputs and outputs double, double accuracy: on the GPU tetrahedra, and
    prisms with two threads per element, compute in 61-bit integers with shared
-   exponents (error against exact results no larger than double arithmetic's) and
-   in double whatever leaves that range; the rest in double throughout.
+   exponents (error against exact results, in the norm of an element's A^e or b^e,
+   no larger than double arithmetic's; entries far below that norm carry its unit)
+   and in double whatever leaves that range; the rest in double throughout.
    FE_FP32_MIXED: coordinates stay double in memory; edge vectors are formed
    exactly enough in single precision, the coefficient and shape-derivative
    arithmetic and accumulation run in float, coefficients and outputs are float.
