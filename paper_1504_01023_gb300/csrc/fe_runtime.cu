@@ -59,15 +59,38 @@ int nc_of(fe_elem_type type, const fe_elem_args *a) {
 }
 static int csize(fe_precision p) { return p == FE_FP32_MIXED ? 4 : 8; }
 
+// Zeroes device memory before it returns, on a stream of its own: a cudaMemset on the
+// default stream is not ordered with the non-blocking streams that use the memory next
+// (side streams, serving slots, the host pipeline), and waits behind what the program
+// has queued there.
+static fe_status zero_now(fe_ctx *ctx, void *p, size_t bytes) {
+    cudaStream_t s = nullptr;
+    cudaError_t e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
+    if (e != cudaSuccess) return cuda_check(ctx, e, "cudaStreamCreate(zero)");
+    e = cudaMemsetAsync(p, 0, bytes, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    cudaStreamDestroy(s);
+    return cuda_check(ctx, e, "zeroing scratch");
+}
+
+// A zeroed device word (64 bytes) at p, allocated once.
+static fe_status ensure_word(fe_ctx *ctx, void **p, const char *what) {
+    if (*p) return FE_OK;
+    void *w = nullptr;
+    fe_status st = ctx_malloc(ctx, &w, 64, what);
+    if (st != FE_OK) return st;
+    st = zero_now(ctx, w, 64);
+    if (st != FE_OK)
+        cudaFree(w);
+    else
+        *p = w;
+    return st;
+}
+
 fe_status ensure_scratch(fe_ctx *ctx, Scratch &s, uint64_t n) {
-    if (!s.fix_count) {
-        fe_status st = ctx_malloc(ctx, reinterpret_cast<void **>(&s.fix_count), 64, "cudaMalloc(fix_count)");
-        if (st != FE_OK) return st;
-        st = ctx_malloc(ctx, reinterpret_cast<void **>(&s.status), 64, "cudaMalloc(status)");
-        if (st != FE_OK) return st;
-        cudaMemset(s.fix_count, 0, 64);
-        cudaMemset(s.status, 0, 64);
-    }
+    fe_status w = ensure_word(ctx, reinterpret_cast<void **>(&s.fix_count), "cudaMalloc(fix_count)");
+    if (w == FE_OK) w = ensure_word(ctx, reinterpret_cast<void **>(&s.status), "cudaMalloc(status)");
+    if (w != FE_OK) return w;
     if (n > 0xFFFFFFFFull) return set_error(ctx, FE_ERR_INVALID_ARG, "more than 2^32-1 elements in one call");
     if (n > s.fix_cap) {
         if (s.fix_list) cudaFree(s.fix_list);
@@ -851,7 +874,8 @@ fe_status fe_ctx_sync(fe_ctx *ctx) {
         cudaMemcpy(ctx->h_status, ctx->scratch.status, sizeof(int), cudaMemcpyDeviceToHost);
         const int s = *ctx->h_status;
         if (s) {
-            cudaMemset(ctx->scratch.status, 0, sizeof(int));
+            const fe_status z = zero_now(ctx, ctx->scratch.status, sizeof(int));
+            if (z != FE_OK) return z;
             if (s & ST_TMA_TIMEOUT) return set_error(ctx, FE_ERR_TIMEOUT, "a bulk copy wait ran out");
             if (s & ST_SKIPPED_TILES)
                 return set_error(ctx, FE_ERR_PARTIAL, "tiles were skipped (injected fault): outputs incomplete");
