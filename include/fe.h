@@ -32,6 +32,12 @@
  *  - A context is used by one host thread at a time, except fe_serve_submit,
  *    fe_serve_poll, fe_serve_wait_any and fe_serve_release, which may be called
  *    from any thread.
+ *  - Calls of a context on different streams may overlap on the device. Each of the 16
+ *    streams used last has a fix-up list of its own; a call on a further stream takes
+ *    over the oldest one's, behind that stream's last call. Calls captured in CUDA
+ *    graphs share one list of the context, apart from the streams': their replays may
+ *    overlap plain calls, but two replays, or parallel branches, with FE_FP32_MIXED or
+ *    FE_FP64_DW calls of one context must not overlap each other.
  */
 #ifndef FE_H_
 #define FE_H_
@@ -196,8 +202,8 @@ typedef struct fe_out {
     int packed;                    /* 1: upper triangle of a symmetric A^e (FE_POISSON) */
 } fe_out;
 
-/* Create a context on cfg->device (NULL cfg = device 0, defaults). Allocates the
-   context's scratch (fix-up lists, status words) and streams. */
+/* Create a context on cfg->device (NULL cfg = device 0, defaults). Its scratch (fix-up
+   lists, status word) is allocated here and by the first calls that need it. */
 fe_status fe_ctx_create(const fe_ctx_config *cfg, fe_ctx **out);
 /* Stop serving, free every resident mesh, output and scratch buffer. */
 fe_status fe_ctx_destroy(fe_ctx *ctx);

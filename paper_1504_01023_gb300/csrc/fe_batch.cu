@@ -213,7 +213,7 @@ static fe_status launch_class(fe_ctx *ctx, BatchPlan *pl, const ClassLaunch &cl,
         if (e == cudaSuccess) e = cudaMemsetAsync(pl->scratch.fix_count, 0, sizeof(unsigned), s);
         if (e != cudaSuccess) return cuda_check(ctx, e, "cudaMemsetAsync(batch class)");
     }
-    int *status = ctx->scratch.status;
+    int *status = ctx->status;
     const BatchSeg *segs = pl->d_segs + cl.seg_off;
     unsigned n_segs = cl.n_segs, n_tiles = cl.n_tiles;
     unsigned *counter = cl.persistent ? pl->d_counter + cl.combo : nullptr;
@@ -236,7 +236,7 @@ static fe_status enqueue_batch(fe_ctx *ctx, BatchPlan *pl, cudaStream_t st, bool
         if (e == cudaSuccess) e = cudaMemsetAsync(pl->scratch.fix_count, 0, sizeof(unsigned), st);
         if (e != cudaSuccess) return cuda_check(ctx, e, "cudaMemsetAsync(batch)");
     }
-    int *status = ctx->scratch.status;
+    int *status = ctx->status;
     const bool fork = branches && pl->classes.size() > 1;
     BatchCache *bc = ctx->batch;
     if (fork) {
@@ -302,7 +302,7 @@ static fe_status build_plan(fe_ctx *ctx, const fe_batch_item *items, int n, size
         d.p.fix_count = pl->scratch.fix_count;
         d.p.fix_cap = pl->scratch.fix_cap;
         d.p.item = unsigned(i);
-        d.p.status = ctx->scratch.status;
+        d.p.status = ctx->status;
         d.combo = batch_combo(items[i].type, a.kind, a.quad, a.coef_mode == FE_COEF_PER_QPOINT);
     }
     if (st == FE_OK) {
@@ -459,7 +459,7 @@ fe_status dyn_batch_launch(fe_ctx *ctx, DynBatch &db, std::vector<BatchItemDev> 
         it.p.fix_list = db.scratch.fix_list;
         it.p.fix_count = d_fix_count;
         it.p.fix_cap = db.scratch.fix_cap;
-        it.p.status = ctx->scratch.status;
+        it.p.status = ctx->status;
     }
     memset(db.h_tab, 0, kItemsOff);
     memcpy(db.h_tab + kItemsOff, items.data(), items.size() * sizeof(BatchItemDev));

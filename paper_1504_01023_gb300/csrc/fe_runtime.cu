@@ -89,7 +89,6 @@ static fe_status ensure_word(fe_ctx *ctx, void **p, const char *what) {
 
 fe_status ensure_scratch(fe_ctx *ctx, Scratch &s, uint64_t n) {
     fe_status w = ensure_word(ctx, reinterpret_cast<void **>(&s.fix_count), "cudaMalloc(fix_count)");
-    if (w == FE_OK) w = ensure_word(ctx, reinterpret_cast<void **>(&s.status), "cudaMalloc(status)");
     if (w != FE_OK) return w;
     if (n > 0xFFFFFFFFull) return set_error(ctx, FE_ERR_INVALID_ARG, "more than 2^32-1 elements in one call");
     if (n > s.fix_cap) {
@@ -108,8 +107,57 @@ fe_status ensure_scratch(fe_ctx *ctx, Scratch &s, uint64_t n) {
 void free_scratch(Scratch &s) {
     if (s.fix_list) cudaFree(s.fix_list);
     if (s.fix_count) cudaFree(s.fix_count);
-    if (s.status) cudaFree(s.status);
     s = Scratch{};
+}
+
+// The scratch of calls captured in a graph, for n elements. It is apart from the
+// streams': a replay may run on any stream, beside their calls. Allocation is allowed
+// in the capture; an outgrown list stays for the graphs that write to it (the list at
+// least doubles, so these take less than it does).
+static fe_status captured_scratch(fe_ctx *ctx, uint64_t n) {
+    Scratch &c = ctx->captured;
+    if (c.fix_count && n <= c.fix_cap) return FE_OK;
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    Scratch grown;
+    grown.fix_count = c.fix_count;
+    const uint64_t twice = std::min<uint64_t>(2 * uint64_t(c.fix_cap), 0xFFFFFFFFull);
+    const fe_status st = ensure_scratch(ctx, grown, std::max(n, twice));
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (st == FE_OK && c.fix_list) ctx->captured_old.push_back(c.fix_list);
+    if (st == FE_OK) c = grown;
+    else c.fix_count = grown.fix_count;
+    return st;
+}
+
+// The scratch of plain calls on stream st, for n elements.
+static fe_status stream_scratch(fe_ctx *ctx, cudaStream_t st, uint64_t n, StreamScratch *&out) {
+    unsigned long long id = 0;
+    const cudaError_t ce = cudaStreamGetId(st, &id);
+    if (ce != cudaSuccess) return cuda_check(ctx, ce, "cudaStreamGetId");
+    out = nullptr;
+    StreamScratch *oldest = nullptr;
+    for (StreamScratch &e : ctx->scratch) {
+        if (e.id == id) out = &e;
+        if (!oldest || e.last < oldest->last) oldest = &e;
+    }
+    if (!out && ctx->scratch.size() < kStreamScratch) {
+        StreamScratch e;
+        e.id = id;
+        const cudaError_t ee = cudaEventCreateWithFlags(&e.done, cudaEventDisableTiming);
+        if (ee != cudaSuccess) return cuda_check(ctx, ee, "cudaEventCreate(scratch)");
+        ctx->scratch.push_back(e);
+        out = &ctx->scratch.back();
+    } else if (!out) {
+        // calls record `done` once the streams are this many (launch_set): before that
+        // the whole device is waited for, once per scratch
+        const cudaError_t we = oldest->recorded ? cudaStreamWaitEvent(st, oldest->done, 0) : cudaDeviceSynchronize();
+        if (we != cudaSuccess) return cuda_check(ctx, we, "scratch of another stream");
+        out = oldest;
+        out->id = id;
+    }
+    out->last = ++ctx->scratch_calls;
+    return ensure_scratch(ctx, out->s, n);
 }
 
 // Kernel template value of the coefficient mode: 0 per element, 1 per point,
@@ -350,7 +398,7 @@ static cudaError_t launch_dependent(const void *k, int64_t grid, int threads, vo
     return cudaLaunchKernelExC(&cfg, k, args);
 }
 
-fe_status launch_set(fe_ctx *ctx, fe_elem_type type, const fe_elem_args *a, const fe_out *o, Scratch &s, cudaStream_t st,
+fe_status launch_set(fe_ctx *ctx, fe_elem_type type, const fe_elem_args *a, const fe_out *o, Scratch *own, cudaStream_t st,
                      const Shape *force, const void *x, bool mapped) {
     if (a->n_elem == 0) return FE_OK;
     const int outl = out_mode(o);
@@ -429,17 +477,32 @@ fe_status launch_set(fe_ctx *ctx, fe_elem_type type, const fe_elem_args *a, cons
         if (ctx->skip_launches.fetch_sub(1) > 0) p.skip_mod = ctx->skip_mod;
     }
     const bool fixup = a->prec != FE_FP64;   // mixed and double-word forms flag elements
+    StreamScratch *ss = nullptr;
     if (fixup) {
-        fe_status e = ensure_scratch(ctx, s, uint64_t(a->n_elem));
+        const uint64_t n = uint64_t(a->n_elem);
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        // (an error: the default stream while a blocking stream is captured; the launch reports it)
+        if (!own && cudaStreamIsCapturing(st, &cap) != cudaSuccess) cudaGetLastError();
+        const Scratch *s = own;
+        fe_status e;
+        if (own) {
+            e = ensure_scratch(ctx, *own, n);
+        } else if (cap != cudaStreamCaptureStatusNone) {
+            e = captured_scratch(ctx, n);
+            s = &ctx->captured;
+            // each replay zeroes the counter, whatever replays of other graphs left
+            if (e == FE_OK)
+                e = cuda_check(ctx, cudaMemsetAsync(s->fix_count, 0, 2 * sizeof(unsigned), st), "cudaMemsetAsync(captured)");
+        } else {
+            e = stream_scratch(ctx, st, n, ss);
+            if (ss) s = &ss->s;
+        }
         if (e != FE_OK) return e;
-        p.fix_list = s.fix_list;
-        p.fix_count = s.fix_count;
-        p.fix_cap = s.fix_cap;
-    } else if (!s.status) {
-        fe_status e = ensure_scratch(ctx, s, 0);
-        if (e != FE_OK) return e;
+        p.fix_list = s->fix_list;
+        p.fix_count = s->fix_count;
+        p.fix_cap = s->fix_cap;
     }
-    p.status = s.status;
+    p.status = ctx->status;
 
     CoefFn fn;
     memset(&fn, 0, sizeof fn);
@@ -478,10 +541,11 @@ fe_status launch_set(fe_ctx *ctx, fe_elem_type type, const fe_elem_args *a, cons
         void *fargs[] = {&p, &fn};
         ce = launch_dependent(fk, std::max<int64_t>(fgrid, 1), 256, fargs, 0, st);
         if (ce != cudaSuccess) {
-            cudaMemsetAsync(s.fix_count, 0, 2 * sizeof(unsigned), st);   // what the fix-up would have left
+            cudaMemsetAsync(p.fix_count, 0, 2 * sizeof(unsigned), st);   // what the fix-up would have left
             return cuda_check(ctx, ce, "cudaLaunchKernel(fixup)");
         }
         g_launches.fetch_add(1, std::memory_order_relaxed);
+        if (ss && ctx->scratch.size() == kStreamScratch) ss->recorded = cudaEventRecord(ss->done, st) == cudaSuccess;
     }
     return FE_OK;
 }
@@ -598,7 +662,7 @@ static fe_status host_pipeline(fe_ctx *ctx, fe_elem_type type, const fe_elem_arg
             co.flags = o->flags ? o->flags + c0 : nullptr;
         }
         if (co.layout == FE_LAYOUT_SOA && out_host) co.stride = K;
-        result = launch_set(ctx, type, &ca, &co, ctx->scratch, ctx->s_comp);
+        result = launch_set(ctx, type, &ca, &co, nullptr, ctx->s_comp);
         cudaEventRecord(comp_done[slot], ctx->s_comp);
         if (out_host) {
             cudaStreamWaitEvent(ctx->s_out, comp_done[slot], 0);
@@ -661,7 +725,7 @@ static bool zero_copy(fe_ctx *ctx, fe_elem_type type, const fe_elem_args *a, con
         if (!dout.A || !dout.b || (o->flags && !dout.flags)) return false;
         dout.memory = FE_MEM_DEVICE;
     }
-    st = launch_set(ctx, type, &da, &dout, ctx->scratch, s, nullptr, nullptr, true);
+    st = launch_set(ctx, type, &da, &dout, nullptr, s, nullptr, nullptr, true);
     if (st == FE_OK) st = cuda_check(ctx, cudaStreamSynchronize(s), "zero-copy integration");
     return true;
 }
@@ -686,7 +750,7 @@ static fe_status integrate(fe_ctx *ctx, fe_elem_type type, const fe_elem_args *a
         st = fe_tune(ctx, type, a, o, stream);
         if (st != FE_OK) return st;
     }
-    return launch_set(ctx, type, a, o, ctx->scratch, s);
+    return launch_set(ctx, type, a, o, nullptr, s);
 }
 
 static void load_tuning_cache(fe_ctx *ctx) {
@@ -829,7 +893,7 @@ fe_status fe_ctx_create(const fe_ctx_config *cfg, fe_ctx **out) {
     ctx->serve_slots = c.serve_slots > 0 ? std::min(c.serve_slots, 64) : 4;
     if (c.tuning_cache_path) ctx->tuning_cache_path = c.tuning_cache_path;
     load_tuning_cache(ctx);
-    fe_status st = ensure_scratch(ctx, ctx->scratch, 0);
+    fe_status st = ensure_word(ctx, reinterpret_cast<void **>(&ctx->status), "cudaMalloc(status)");
     if (st != FE_OK) {
         delete ctx;
         return st;
@@ -845,7 +909,13 @@ fe_status fe_ctx_destroy(fe_ctx *ctx) {
     serve_destroy(ctx);
     batch_destroy(ctx);
     cudaDeviceSynchronize();
-    free_scratch(ctx->scratch);
+    for (StreamScratch &e : ctx->scratch) {
+        free_scratch(e.s);
+        cudaEventDestroy(e.done);
+    }
+    free_scratch(ctx->captured);
+    for (void *p : ctx->captured_old) cudaFree(p);
+    if (ctx->status) cudaFree(ctx->status);
     for (auto &kv : ctx->meshes) cudaFree(kv.second.coords);
     for (int s = 0; s < 2; ++s)
         for (int i = 0; i < 5; ++i)
@@ -870,11 +940,11 @@ fe_status fe_ctx_sync(fe_ctx *ctx) {
     cudaSetDevice(ctx->device);
     cudaError_t e = cudaDeviceSynchronize();
     if (e != cudaSuccess) return cuda_check(ctx, e, "device synchronize");
-    if (ctx->scratch.status) {
-        cudaMemcpy(ctx->h_status, ctx->scratch.status, sizeof(int), cudaMemcpyDeviceToHost);
+    if (ctx->status) {
+        cudaMemcpy(ctx->h_status, ctx->status, sizeof(int), cudaMemcpyDeviceToHost);
         const int s = *ctx->h_status;
         if (s) {
-            const fe_status z = zero_now(ctx, ctx->scratch.status, sizeof(int));
+            const fe_status z = zero_now(ctx, ctx->status, sizeof(int));
             if (z != FE_OK) return z;
             if (s & ST_TMA_TIMEOUT) return set_error(ctx, FE_ERR_TIMEOUT, "a bulk copy wait ran out");
             if (s & ST_SKIPPED_TILES)
@@ -939,7 +1009,7 @@ static fe_status apply(fe_ctx *ctx, fe_elem_type type, const fe_elem_args *a, co
     // kernels unless fe_set_shape chose one
     const std::string key = shape_key(type, a, &o);
     if (!ctx->shapes.count(key)) ctx->shapes[key] = Shape{64, 1};
-    return launch_set(ctx, type, a, &o, ctx->scratch, static_cast<cudaStream_t>(stream), nullptr, x);
+    return launch_set(ctx, type, a, &o, nullptr, static_cast<cudaStream_t>(stream), nullptr, x);
 }
 
 fe_status fe_apply_tet(fe_ctx *ctx, const fe_elem_args *args, const void *x, void *y, void *f, uint8_t *flags,
@@ -982,7 +1052,7 @@ fe_status fe_selftest_bounded_wait(fe_ctx *ctx, unsigned polls, void *stream) {
     if (polls == 0 || polls > (1u << 22)) return set_error(ctx, FE_ERR_INVALID_ARG, "polls must be in [1, 2^22]");
     cudaSetDevice(ctx->device);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    int *status = ctx->scratch.status;
+    int *status = ctx->status;
     void *args[] = {&polls, &status};
     cudaError_t e = cudaLaunchKernel(kernel_selftest_wait(), dim3(1), dim3(32), args, 0, s);
     if (e != cudaSuccess) return cuda_check(ctx, e, "cudaLaunchKernel(selftest)");
@@ -1111,11 +1181,11 @@ fe_status fe_tune(fe_ctx *ctx, fe_elem_type type, const fe_elem_args *a, const f
     }
     for (const Shape &sh : cands) {
         if (smem_bytes(type, a, out_mode(o), sh.block, sh.tpe) + kStaticSmem > ctx->max_smem_optin) continue;
-        st = launch_set(ctx, type, a, o, ctx->scratch, s, &sh);  // warm-up
+        st = launch_set(ctx, type, a, o, nullptr, s, &sh);  // warm-up
         if (st != FE_OK) break;
         cudaEventRecord(e0, s);
         const int reps = 3;
-        for (int r = 0; r < reps && st == FE_OK; ++r) st = launch_set(ctx, type, a, o, ctx->scratch, s, &sh);
+        for (int r = 0; r < reps && st == FE_OK; ++r) st = launch_set(ctx, type, a, o, nullptr, s, &sh);
         cudaEventRecord(e1, s);
         if (st != FE_OK) break;
         cudaError_t ce = cudaEventSynchronize(e1);

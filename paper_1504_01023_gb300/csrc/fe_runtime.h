@@ -31,13 +31,27 @@ struct TraceRange {
 
 extern std::atomic<uint64_t> g_launches;
 
-// Device scratch of one launch sequence (fix-up list, its counter, status word).
+// Device scratch of one launch sequence: the fix-up list and its counter, which each
+// call finds at zero and leaves at zero (fixup_kernel).
 struct Scratch {
     unsigned long long *fix_list = nullptr;
     unsigned int fix_cap = 0;
     unsigned int *fix_count = nullptr;
-    int *status = nullptr;
 };
+
+// The scratch of plain calls on one stream. Calls on different streams may overlap:
+// on a shared counter their lists would mix, and the last block of a fix-up, which
+// sets the counter back, could not be told.
+struct StreamScratch {
+    unsigned long long id = 0;      // cudaStreamGetId: unique, unlike a handle that is used again
+    uint64_t last = 0;              // number of its last call
+    bool recorded = false;          // `done` follows that call
+    cudaEvent_t done = nullptr;
+    Scratch s;
+};
+// Streams with a scratch of their own; a further one takes over the least recently used
+// one's, behind its last call.
+constexpr size_t kStreamScratch = 16;
 
 struct Shape {
     int block = 0;          // elements per tile
@@ -68,7 +82,11 @@ struct fe_ctx {
     std::mutex err_mu;
     fe_status async_error = FE_OK;
 
-    fe::Scratch scratch;            // plain calls
+    int *status = nullptr;          // device status word of every launch
+    std::vector<fe::StreamScratch> scratch;   // plain calls, by stream
+    uint64_t scratch_calls = 0;
+    fe::Scratch captured;           // calls captured in a graph
+    std::vector<void *> captured_old;         // its outgrown lists: graphs hold their addresses
     int *h_status = nullptr;        // pinned mirror for status reads
 
     // profiling
@@ -118,12 +136,13 @@ fe_status ctx_malloc(fe_ctx *ctx, void **p, size_t bytes, const char *what);
 bool take_alloc_fault(fe_ctx *ctx);
 fe_status ensure_scratch(fe_ctx *ctx, Scratch &s, uint64_t n);
 void free_scratch(Scratch &s);
-// Launch main + fix-up kernels of one homogeneous set (device pointers).
+// Launch main + fix-up kernels of one homogeneous set (device pointers), with the
+// scratch `own` (one stream's, outside of captures) or else the stream's.
 // With `force`, that launch shape is used and the context's tuned shapes and
 // profiling events are not touched (safe from the serving thread).
 // x: the nodal input vector of the matrix-free output mode (fe_apply_*).
 // mapped: buffers are host memory through its mapped addresses.
-fe_status launch_set(fe_ctx *ctx, fe_elem_type type, const fe_elem_args *a, const fe_out *o, Scratch &s,
+fe_status launch_set(fe_ctx *ctx, fe_elem_type type, const fe_elem_args *a, const fe_out *o, Scratch *own,
                      cudaStream_t st, const Shape *force = nullptr, const void *x = nullptr, bool mapped = false);
 Shape default_shape(fe_elem_type type);
 // Dynamically built batch (serving): device tables grown on demand, uploaded

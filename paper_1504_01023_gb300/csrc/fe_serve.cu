@@ -215,7 +215,7 @@ static void launch_jobs(ServeState *s, Slot &sl, std::vector<Job> &jobs) {
             // pipe; 300,000 generic per point 990 -> 240 us a call, Laplace 309 -> 106,
             // 300 elements 64 -> 15)
             const Shape sh = m.type == FE_PRISM && a.prec == FE_FP64 ? Shape{32, 0, 2} : default_shape(m.type);
-            j.status = launch_set(ctx, m.type, &a, &o, sl.plain, sl.stream, &sh);
+            j.status = launch_set(ctx, m.type, &a, &o, &sl.plain, sl.stream, &sh);
         }
     }
     if (!items.empty()) {

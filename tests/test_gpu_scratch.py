@@ -1,6 +1,7 @@
 """The scratch of mixed and double-word calls (list and counter of the elements for the
-double Jacobian pass) on the stream of the call: first calls of a context and of its
-serving slots beside a default stream that is still busy, against the oracle."""
+double Jacobian pass) on the stream of the call, against the oracle: first calls of a
+context and of its serving slots beside a default stream that is still busy; calls and
+replays that overlap on several streams, and the calls that follow them alone."""
 import time
 
 import numpy as np
@@ -80,3 +81,80 @@ def test_first_served_requests_beside_a_busy_default_stream():
             ctx.serve_release(t)
         ctx.mesh_release(mid)
         ctx.sync()
+
+
+def _alone(ctx, cases):
+    """Calls with nothing else on the device, and a matrix-free product (which adds an
+    element twice if its fix-up list holds entries of an earlier call)."""
+    for case in cases:
+        for t in case.out:
+            t.zero_()
+        case.call(ctx)
+        ctx.sync()
+        case.check()
+        n, (Ao, bo) = case.n, case.ref
+        nodes = case.X.reshape(-1, 3)
+        conn = torch.arange(4 * n, dtype=torch.int32, device="cuda").reshape(n, 4)
+        dt = torch.float32 if case.prec == api.FP32_MIXED else torch.float64
+        y, f = torch.zeros(4 * n, dtype=dt, device="cuda"), torch.zeros(4 * n, dtype=dt, device="cuda")
+        ctx.apply(api.TET, nodes, conn, case.C, api.GENERIC, api.QUAD_TET4, torch.ones_like(y), y, f, prec=case.prec)
+        ctx.sync()
+        # row sums of A: four entries, each within the form's tolerance of the element's norm
+        ey = np.abs(y.cpu().numpy().reshape(n, 4) - Ao.sum(2)).max(1) / np.linalg.norm(Ao, axis=(1, 2))
+        assert ey.max() <= 4 * TOL[case.prec]
+        assert max_errors(Ao, f.cpu().numpy().reshape(n, 4).astype(np.float64), Ao, bo)[1] <= TOL[case.prec]
+
+
+@pytest.mark.parametrize("prec", [api.FP32_MIXED, api.FP64_DW])
+def test_calls_overlapping_on_two_streams(prec):
+    cases = [Case(20001, prec, 31), Case(1003, prec, 32)]
+    streams = [torch.cuda.Stream() for _ in cases]
+    torch.cuda.synchronize()
+    with api.Context(0) as ctx:
+        for _ in range(100):
+            for case, s in zip(cases, streams):
+                case.call(ctx, s)
+        torch.cuda.synchronize()
+        for case in cases:
+            case.check()
+        _alone(ctx, cases)
+
+
+@pytest.mark.parametrize("prec", [api.FP32_MIXED, api.FP64_DW])
+def test_replays_overlapping_plain_calls(prec):
+    captured, plain = Case(20001, prec, 41), Case(1003, prec, 42)
+    larger = Case(24000, prec, 43)       # its capture outgrows the first graph's list
+    s, t = torch.cuda.Stream(), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with api.Context(0) as ctx:
+        graphs = []
+        for case in (captured, larger):
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g, stream=s):
+                case.call(ctx, s)
+                case.call(ctx, s)
+            graphs.append(g)
+        for _ in range(50):
+            with torch.cuda.stream(s):
+                for g in graphs:
+                    g.replay()
+            plain.call(ctx, t)
+            plain.call(ctx, t)
+        torch.cuda.synchronize()
+        for case in (captured, larger, plain):
+            case.check()
+        _alone(ctx, [plain, captured])
+
+
+def test_more_streams_than_scratch():
+    cases = [Case(500 + 211 * i, api.FP32_MIXED, 50 + i) for i in range(24)]
+    streams = [torch.cuda.Stream() if i % 3 else torch.cuda.Stream(priority=-1) for i in range(24)]
+    torch.cuda.synchronize()
+    with api.Context(0) as ctx:
+        for order in (range(24), reversed(range(24)), range(0, 24, 2)):
+            for i in order:
+                cases[i].call(ctx, streams[i])
+        torch.cuda.synchronize()
+        for case in cases:
+            case.check()
+        _alone(ctx, cases[:2])
