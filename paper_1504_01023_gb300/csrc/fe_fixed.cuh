@@ -240,9 +240,9 @@ template <class S> FE_HD void fx_quad(const S &s, int j, double v[4]) {
 // D = diag(2^X) over the axes' cofactors and t, (a_r, t) = a^_r D and the integers
 // a^_r meet the coefficients D C^ D, which share one exponent per element.
 //
-// False (nothing written) for elements that the double form takes: exponents of
-// the edges or of the results outside the windows below (infinities and NaN among
-// them), det J below 2^-20 of |edge| |cofactor| after that scaling (nearly or
+// False (nothing written) for elements that the double form takes: exponents of the
+// edges or of the results outside the windows below (infinities and NaN among them),
+// det J below 2^-20 of |edge| |cofactor| after that scaling (nearly or
 // exactly degenerate: its sign and the degeneracy test are then those of the
 // double form) or all cofactors below 2^-8 of |edge|^2 (nearly parallel edges).
 struct TetFx {
@@ -251,6 +251,16 @@ struct TetFx {
     // results within 2^-700 .. 2^600 (of their last bit) then exclude an infinite or
     // NaN coefficient (2^1024 and more) and admit any within 2^+-300.
     static constexpr int kEdgeWin = 80, kLow = -700, kHigh = 600;
+    // Evenness: an element's results share a unit (that of the largest), where double
+    // gives every product its own. The kernels leave elements to the double form in which
+    // this could cost more than double's own cancellation: generic ones whose weighted
+    // diagonal diffusion coefficients that are not zero spread over more than
+    // kDiagSpread + 1 bits (anisotropic diffusion along the axes, flat elements). 10,368
+    // jittered tetrahedra with diffusion diag(1, e, e), 99% point of the largest relative
+    // error of an entry of A^e, fixed / double: e = 2^-4 0.30, 2^-8 0.70, 2^-10 1.4, 2^-12 2.2,
+    // 2^-20 33; with full random coefficients and the z axis scaled by 2^-3 1.05, 2^-5 3.4.
+    // With the benchmark's coefficients one in 50,000 is left.
+    static constexpr int kDiagSpread = 7;
     FE_HD static bool outside(int x) { return static_cast<unsigned>(x - kLow) > static_cast<unsigned>(kHigh - kLow); }
 
     Fx2 a[3][3];        // cofactor rows 1..3, exponents X[0..2] along the axes
@@ -365,6 +375,18 @@ struct TetFx {
 #pragma unroll
         for (int s = 0; s < 3; ++s) A[1 + s] = A[4 * (1 + s)] = fx_to(row0[s], xo);
         A[0] = fx_to(-(row0[0] + row0[1] + row0[2]), xo);
+    }
+
+    // Generic kind: see kDiagSpread. (A zero's exponent field is 0: never the largest.)
+    template <class CS> FE_HD bool even(const CS &c) const {
+        int mn = 1 << 20, mx = -(1 << 20);
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            const int f = fx_exp(c(5 + 5 * i)), e = f + 2 * X[i];
+            mn = fx_mini(mn, f ? e : 1 << 20);
+            mx = fx_maxi(mx, e);
+        }
+        return mx - mn <= kDiagSpread;
     }
 
     // Generic kind, MASS2: the four-point rule (kappa = 0.8, mass term twice on the

@@ -83,7 +83,7 @@ template <int KIND, int QUAD, int CPQ> struct ElemMath<TET, KIND, FP64, QUAD, CP
                     fx.laplace(A);
                     poisson_b(fx.volume(), c, b);
                 } else {
-                    ok = fx.template generic<QUAD == Q_TET4>(c, A, b);
+                    ok = fx.even(c) && fx.template generic<QUAD == Q_TET4>(c, A, b);
                 }
                 if (ok) return fx.neg ? 2 : 0;
             }
@@ -877,7 +877,7 @@ template <int KIND, int CPQ> struct ElemMath<PRISM, KIND, FP64, Q_PRISM6, CPQ> {
         b3 |= __shfl_xor_sync(mask, b3, 1);
         uint32_t d = P.set_a(b12, b3);
         P.set_det(d | __shfl_xor_sync(mask, d, 1));
-        P.template exponents<KIND>(cl, NP);
+        P.template exponents<KIND, true>(cl, NP);
 #pragma unroll
         for (int j = KIND == POISSON ? 5 : 0; j < 6; ++j) P.En[j] = max(P.En[j], __shfl_xor_sync(mask, P.En[j], 1));
         P.template common_exponents<KIND>();

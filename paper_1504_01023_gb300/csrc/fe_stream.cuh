@@ -138,7 +138,7 @@ template <int KIND, int QUAD, int CPQ> __device__ __forceinline__ void stream_ti
                 if constexpr (KIND == POISSON)
                     EM::poisson_b(fx.volume(), cs, b);
                 else
-                    ok = fx.template columns<MASS2>(cs, R, b);
+                    ok = fx.even(cs) && fx.template columns<MASS2>(cs, R, b);
             }
             if (ok) {
                 st_row4(Bout + e * 4, b, o32);
