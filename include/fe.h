@@ -69,10 +69,15 @@ typedef enum fe_elem_type { FE_TET = 0, FE_PRISM = 1 } fe_elem_type;
 typedef enum fe_problem { FE_POISSON = 0, FE_GENERIC = 1 } fe_problem;
 
 /* FE_FP64: inputs and outputs double, double accuracy: on the GPU tetrahedra, and
-   prisms with two threads per element, compute in 61-bit integers with shared
-   exponents (error against exact results, in the norm of an element's A^e or b^e,
-   no larger than double arithmetic's; entries far below that norm carry its unit)
-   and in double whatever leaves that range; the rest in double throughout.
+   prisms with two threads per element, compute in 61-bit integers with exponents
+   shared by an element, and in double the elements in which these could cost
+   accuracy: strongly anisotropic diffusion along the axes, edges of very different
+   lengths, nearly degenerate ones, values outside the integers' range. Against exact
+   results, in the norm of an element's A^e or b^e, the errors over a mesh are then
+   about half of double arithmetic's on jittered meshes and within a bit of them on
+   the stretched, sheared, flat and tall ones measured; an entry down to 2^-8 of the
+   largest keeps about ten times double's relative error at most. The rest is in
+   double throughout.
    FE_FP32_MIXED: coordinates stay double in memory; edge vectors are formed
    exactly enough in single precision, the coefficient and shape-derivative
    arithmetic and accumulation run in float, coefficients and outputs are float.

@@ -77,10 +77,10 @@ template <int KIND, int QUAD, int CPQ> struct ElemMath<TET, KIND, FP64, QUAD, CP
             return is_neg(geo.det) ? 2 : 0;
         } else {
             TetFx fx;
-            if (fx.geometry(x)) {
+            if (fx.geometry(x) && fx.even_rows()) {
                 bool ok = true;
                 if constexpr (KIND == POISSON) {
-                    fx.laplace(A);
+                    ok = fx.laplace(A);
                     poisson_b(fx.volume(), c, b);
                 } else {
                     ok = fx.even(c) && fx.template generic<QUAD == Q_TET4>(c, A, b);
@@ -889,6 +889,7 @@ template <int KIND, int CPQ> struct ElemMath<PRISM, KIND, FP64, Q_PRISM6, CPQ> {
             if (t == 0) {
                 T12 = max(T12, __shfl_xor_sync(mask, T12, 1));
                 P.set_products(T12, max(T3, __shfl_xor_sync(mask, T3, 1)));
+                if (KIND == GENERIC) P.ok = P.ok && P.even_shape();
             }
             P.template gamma<KIND>(t);
         }

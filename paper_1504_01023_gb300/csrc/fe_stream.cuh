@@ -133,7 +133,7 @@ template <int KIND, int QUAD, int CPQ> __device__ __forceinline__ void stream_ti
         if (active) {
             const RecSrc<12> xs{sX + lane * 12};
             const RecSrc<NC> cs{sC + lane * NC};
-            ok = fx.geometry(xs);
+            ok = fx.geometry(xs) && fx.even_rows();
             if (ok) {
                 if constexpr (KIND == POISSON)
                     EM::poisson_b(fx.volume(), cs, b);
@@ -153,7 +153,7 @@ template <int KIND, int QUAD, int CPQ> __device__ __forceinline__ void stream_ti
                 double *Ae = Aout + e * 16;
                 if constexpr (KIND == POISSON) {
                     double A[16];
-                    fx.laplace(A);
+                    ok = fx.laplace(A);
 #pragma unroll
                     for (int r = 0; r < 4; ++r) st_row4(Ae + 4 * r, A + 4 * r, o32);
                 } else {
@@ -166,9 +166,8 @@ template <int KIND, int QUAD, int CPQ> __device__ __forceinline__ void stream_ti
                         st_row4(Ae + 4 * r, A, o32);
                     }
                 }
-            } else {
-                stream_double_elem<KIND, QUAD, CPQ>(p, e);
             }
+            if (!ok) stream_double_elem<KIND, QUAD, CPQ>(p, e);   // over what a test after the stores leaves
         }
     }
 }
