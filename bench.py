@@ -14,7 +14,9 @@ poorly shaped elements: main kernel plus fix-up) and in the double-word form
 roofline; and the other workloads (the 48,000-element Poisson set as stated,
 prisms, node tables, batches, serving) under further keys.
 
-Prints one JSON line (rank 0). Under torchrun every rank integrates its own
+Prints one short JSON line (rank 0): the step's keys and the rates of the other
+measurements; the full record, with rooflines and launch shapes, goes to the file
+--record. Under torchrun every rank integrates its own
 seeded mesh of that size on its own GPU (weak scaling, no data-path
 collective; the barrier and the max over ranks are timing only).
 
@@ -80,6 +82,8 @@ def parse():
                          "point); other kinds only for profiling")
     ap.add_argument("--shape", default=None, help="BLOCK,PERSISTENT[,THREADS_PER_ELEMENT]: pin the main kernel's "
                                                   "launch shape instead of autotuning it (profiling)")
+    ap.add_argument("--record", default=os.path.join(ROOT, "bench_record.json"),
+                    help="file for the full record of the run ('' writes none)")
     ap.add_argument("--n-slab", type=int, default=1000,
                     help="squares per axis of the prism slab (2 n^2 elements); smaller only for profiling")
     return ap.parse_args()
@@ -443,6 +447,40 @@ def run_reference(args):
     print(json.dumps(line), flush=True)
 
 
+# The printed line is short: readers keep only the last few kilobytes of a run's output.
+LINE_LIMIT = 2500
+
+
+def summary_line(result, record=None):
+    """The printed line of a run: the step's own keys, the end-to-end and CPU rates whole,
+    and of every other measurement its rates (keys ending in melem_s, or value) and its
+    latencies; the full record goes to the file `record`."""
+    keep = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+            "vs_baseline", "dtype", "data", "config", "gpu_launches", "clocks")
+    line = {k: result[k] for k in keep if k in result}
+    if "e2e" in result:
+        line["e2e"] = {k: v for k, v in result["e2e"].items() if k != "path"}
+    roof = result.get("roofline", {})
+    hbm = roof.get("hbm", roof)
+    line["roofline"] = {"kernel": roof.get("kernel"), "bound": roof.get("bound"), "frac": roof.get("frac"),
+                        "hbm_gbs": hbm.get("achieved"), "hbm_peak_gbs": hbm.get("peak"), "hbm_frac": hbm.get("frac")}
+    if "cpu_baseline" in result:
+        line["cpu_baseline"] = {k: result["cpu_baseline"].get(k) for k in ("value", "unit", "cores", "kind")}
+    others = {}
+    for name, v in result.items():
+        if name not in line and isinstance(v, dict) and isinstance(v.get("value"), (int, float)):
+            others[name] = round(v["value"], 1)
+    served = result.get("serving", {}).get("served", {})
+    for k in ("sustained_melem_s", "p50_ms", "p99_ms"):
+        if k in served:
+            others["served_" + k] = round(served[k], 3)
+    if others:
+        line["other_melem_s_and_ms"] = others
+    if record:
+        line["record"] = os.path.basename(record)
+    return line
+
+
 def aggregate(ms_total, n_per_rank, steps, world, dist=None, device=None):
     """Max of the timed region over ranks (each rank did n_per_rank elements per
     step); returns (ms per step, whole-job Melem/s)."""
@@ -616,7 +654,15 @@ def run_native(args):
     elif rank == 0:
         result["e2e"] = {"value": None, "unit": "Melem/s", "note": "measured at N=1 only"}
     if rank == 0:
-        print(json.dumps(result), flush=True)
+        record = args.record
+        if record:
+            try:
+                with open(record, "w") as f:
+                    json.dump(result, f, indent=1)
+            except OSError as e:
+                print(f"full record not written: {e}", file=sys.stderr)
+                record = None
+        print(json.dumps(summary_line(result, record)), flush=True)
     ctx.close()
     if world > 1:
         dist.destroy_process_group()

@@ -67,3 +67,39 @@ def test_source_hash_ignores_comments_only():
     edited = src.replace("// bound", "// another note").replace("/* body */", "/* the\nbody */")
     assert bench.code_only(src) == bench.code_only(edited)
     assert bench.code_only(src) != bench.code_only(src.replace("p[0] = K", "p[0] = 2 * K"))
+
+
+def test_printed_line_is_short_and_keeps_the_contract():
+    """A full record of tens of kilobytes prints as one short line with every key that a
+    reader of the benchmark needs, parsed from the last line of the output."""
+    long = {"value": 12345.678901234567, "unit": "Melem/s", "roofline": {"note": "n" * 2000}, "workload": "w" * 500}
+    clk = {"sm_mhz": 2070.0, "sm_max_mhz": 2070.0, "reasons": [], "samples": 200, "samples_in_region": 190,
+           "power_w_max": 1034.55}
+    result = {"metric": bench.METRIC, "value": 11196.123456789012, "unit": "Melem/s", "n_gpus": 1, "steps": 8000,
+              "warmup": 20, "ms_per_step": 0.5358832001686096, "higher_is_better": True, "scaling": "weak",
+              "vs_baseline": None, "dtype": "f64", "data": "synthetic",
+              "config": {"workload": bench.WORKLOAD, "n_elem_per_gpu": 6000000, "bytes_per_element": 416,
+                         "launch_shape": bench.shape_dict((512, 1)),
+                         "l2": "inputs larger than L2: 2.50 GB read+written per step per GPU",
+                         "parallelism": "weak: 1 independent mesh(es), one per GPU"},
+              "roofline": {"bound": "alu", "kernel": "k" * 70, "frac": 0.5, "note": "n" * 500,
+                           "hbm": {"achieved": 4657.731384776873, "peak": 6677.2, "frac": 0.6975575667610485}},
+              "gpu_launches": 8000, "clocks": clk,
+              "e2e": {"value": 743.009764138675, "unit": "Melem/s", "h2d_bytes_per_step": 1536000000,
+                      "d2h_bytes_per_step": 966000000, "ms_per_step": 8.07, "steps": 3, "dtype": "f64", "path": "p" * 300},
+              "cpu_baseline": dict(long, cores=16, kind="oracle"),
+              "serving": {"served": {"p50_ms": 0.2, "p99_ms": 0.5, "sustained_melem_s": 900.123}, "plain_fp64": long},
+              "paper_context": {"melem_s": {"x" * 20: 1.0}}}
+    for name in ("mixed_form", "double_word_form", "fp64_forms", "cfg1_stated", "threads_per_element", "prism_form",
+                 "coef_function_form", "packed_form", "ordering_study", "indexed_form", "apply_form", "batched"):
+        result[name] = dict(long)
+    text = json.dumps(bench.summary_line(result, "/somewhere/bench_record.json"))
+    assert len(json.dumps(result)) > 20000 and len(text) <= bench.LINE_LIMIT and "\n" not in text
+    line = json.loads(text)
+    for k in ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+              "vs_baseline", "dtype", "data", "config", "gpu_launches"):
+        assert line[k] == result[k]
+    assert line["clocks"] == clk and line["e2e"]["value"] == result["e2e"]["value"]
+    assert line["e2e"]["h2d_bytes_per_step"] == 1536000000 and line["e2e"]["d2h_bytes_per_step"] == 966000000
+    assert line["other_melem_s_and_ms"]["mixed_form"] == 12345.7
+    assert bench.summary_line({k: result[k] for k in ("metric", "value", "unit")})["value"] == result["value"]
