@@ -758,15 +758,18 @@ static void load_tuning_cache(fe_ctx *ctx) {
     std::ifstream f(ctx->tuning_cache_path);
     std::string line;
     while (std::getline(f, line)) {
-        // device key elements persistent [threads-per-element]
+        // device key elements persistent [threads-per-element [revision]]
         std::istringstream ls(line);
         std::string dev, key;
-        int block = 0, pers = 0, tpe = 1;
+        int block = 0, pers = 0, tpe = 1, rev = 1;
         if (!(ls >> dev >> key >> block >> pers)) continue;
         if (!(ls >> tpe)) tpe = 1;
+        if (!(ls >> rev)) rev = 1;
+        // chosen for earlier FP64 kernels: the tuner, where it is on, chooses again
+        if (rev < kShapeRevision && ctx->autotune && key.find("p0") != std::string::npos) continue;
         if (dev == ctx->device_name && block > 0 && (tpe == 1 || tpe == 2 || tpe == 4 || tpe == 6 || tpe == 16) &&
             shape_threads(block, tpe))
-            ctx->shapes[key] = Shape{block, pers, tpe};
+            ctx->shapes[key] = Shape{block, pers, tpe, rev};
     }
 }
 
@@ -775,7 +778,7 @@ static void save_tuning_cache(fe_ctx *ctx) {
     std::ofstream f(ctx->tuning_cache_path, std::ios::trunc);
     for (auto &kv : ctx->shapes)
         f << ctx->device_name << " " << kv.first << " " << kv.second.block << " " << kv.second.persistent << " "
-          << kv.second.tpe << "\n";
+          << kv.second.tpe << " " << kv.second.revision << "\n";
 }
 
 }  // namespace fe

@@ -53,10 +53,16 @@ struct StreamScratch {
 // one's, behind its last call.
 constexpr size_t kStreamScratch = 16;
 
+// Which kernels a tuned shape was chosen for. 1: FP64 in doubles; 2: FP64 in block fixed
+// point, whose best shapes are others (300,000 Laplace prisms: one thread per element
+// 309 us, two 106; before, one thread was the better one).
+constexpr int kShapeRevision = 2;
+
 struct Shape {
     int block = 0;          // elements per tile
     int persistent = 0;     // 1: grid = SMs x resident blocks, tiles strided
     int tpe = 1;            // threads per element (2: prisms, element-contiguous)
+    int revision = kShapeRevision;
 };
 
 struct ServeState;          // fe_serve.cu
