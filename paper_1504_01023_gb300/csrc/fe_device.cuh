@@ -541,7 +541,9 @@ __device__ __forceinline__ void tet_generic_aug(const V3<T> a3[3], T f, T sm, T 
 // Every choice gives the same bits (the same IEEE operations in the same order).
 // An integer multiplication that meets an operand or a product outside the
 // normal range (zero aside) sets `sp`; the caller then redoes the element with
-// the double pipe, as TetF64 with F64<false> throughout.
+// the double pipe, as TetF64 with F64<false> throughout. The kernels use that one
+// only (elements that TetFx leaves); the integer groups are held to its bits by
+// fe_selftest_f64_int.
 // The arithmetic is that of tet_geometry, recip_scaled and tet_generic_aug /
 // tet_poisson_products, written out with explicit operations.
 // ---------------------------------------------------------------------------

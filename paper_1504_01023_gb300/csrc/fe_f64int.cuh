@@ -2,11 +2,12 @@
 // even), computed with 32-bit integer instructions.
 //
 // This GPU issues double-precision instructions at 2 per clock per SM and
-// integer instructions at 64 per clock per SM per pipe. The FP64 arithmetic in
-// doubles (per-point tetrahedra, one-thread prisms and what leaves the windows of
-// the block fixed point) is bound by the double pipe while the integer pipes idle,
-// so it runs a part of its multiplications and additions here instead. These are the
-// same IEEE operations, not approximations: for normal operands and a normal
+// integer instructions at 64 per clock per SM per pipe. Prisms in doubles (one
+// thread per element, node tables) are bound by the double pipe while the integer
+// pipes idle, so they run a part of their multiplications here instead (mul_off).
+// Tetrahedra in doubles (per-point coefficients, and what the block fixed point
+// leaves) use the double pipe throughout; TetF64 with integer groups serves
+// fe_selftest_f64_int alone. These are the same IEEE operations, not approximations: for normal operands and a normal
 // result the value returned is the correctly rounded product or sum, bit for
 // bit what the double-precision instruction returns; so is the signed zero of a
 // product with a zero operand. Subnormal, infinite and NaN operands, and results
