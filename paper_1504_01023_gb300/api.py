@@ -230,7 +230,7 @@ def make_args(elem_type, coords, coefs, kind, quad, coef_mode, prec, layout, con
         cf = coefs.reshape(-1, n) if coefs.dim() == 1 else coefs
         # size-1 dimensions may report any stride: only a real element axis must be unit-stride
         assert n <= 1 or (coords.stride(1) == 1 and cf.stride(-1) == 1)
-        a.coords_stride = coords.stride(0) if n > 1 else 0
+        a.coords_stride = coords.stride(0) if n else 0
         # a single plane has no plane stride (size-1 dimensions may report any stride)
         a.coefs_stride = cf.stride(0) if cf.shape[0] > 1 else 0
     else:
@@ -294,8 +294,9 @@ def make_out(A, b, flags, out_layout, packed=False):
     stride = 0
     if out_layout == SOA:
         n = A.shape[1]
-        assert n <= 1 or (A.stride(0) == b.stride(0) and A.stride(1) == 1 and b.stride(1) == 1)
-        stride = A.stride(0) if n > 1 else 0
+        assert n <= 1 or (A.stride(1) == 1 and b.stride(1) == 1)
+        assert n == 0 or A.stride(0) == b.stride(0)
+        stride = A.stride(0) if n else 0
     return Out(A.data_ptr(), b.data_ptr(), out_layout, stride, flags.data_ptr() if flags is not None else None, _mem(A),
                1 if packed else 0)
 
