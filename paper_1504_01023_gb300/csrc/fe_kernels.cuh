@@ -1836,7 +1836,9 @@ __device__ __forceinline__ bool process_tile(const ElemParams &p, int64_t e0, in
     // ---- store outputs ----
     fence_proxy_async_smem();
     __syncthreads();
-    if (out_soa(OUTL) && tm && p.tma_out) {
+    // (a tensor copy writes whole 16-byte units: of a last tile that ends inside one it
+    // would overwrite what follows the plane's elements)
+    if (out_soa(OUTL) && tm && p.tma_out && (nb * sizeof(CT)) % 16 == 0) {
         if (threadIdx.x == 0) {
             tma_store_2d(tm->a, int(e0), 0, sA);
             tma_store_2d(tm->b, int(e0), 0, sB);
