@@ -4,9 +4,9 @@
 #include "fe_stream.cuh"
 
 namespace fe {
-// The tile kernel, or null where plane_kernel always runs (plane_always).
+// The tile kernel, or null where plane_kernel always runs, on host memory too.
 template <int ET, int KIND, int PREC, int QUAD, int CPQ, int INL, int OUTL> const void *tile_kernel() {
-    if constexpr (INL == SOA && out_soa(OUTL) && plane_always(ET, KIND, PREC, CPQ))
+    if constexpr (INL == SOA && out_soa(OUTL) && plane_mapped(ET, KIND, PREC, CPQ))
         return nullptr;
     else
         return reinterpret_cast<const void *>(&elem_kernel<ET, KIND, PREC, QUAD, CPQ, INL, OUTL>);

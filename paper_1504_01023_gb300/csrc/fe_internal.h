@@ -109,6 +109,15 @@ constexpr bool plane_always(int type, int kind, int prec, int cpq) {
     return type == TET ? prec == FP64 || (prec == MIXED && kind == GENERIC)
                        : prec == FP64 || (prec == MIXED && (kind == POISSON || cpq == 0));
 }
+// Those of them that take the same kernels on pinned host memory, where a tensor copy of
+// a tile crosses the host link in longer runs. Tensor copies / straight, ms: 2M FP64 tets
+// generic 2.65 / 2.97, 300k 0.48 / 0.54; 200k mixed tets generic 0.213 / 0.226 (2M 1.78 /
+// 1.79); 400k mixed prisms Laplace 0.50 / 0.55: tiles. 2M FP64 tets Laplace 1.89 / 1.87, 200k
+// 0.257 / 0.236; FP64 prisms 400k generic per element 1.23 / 0.85, Laplace 0.88 / 0.81; 400k
+// mixed prisms generic per element 0.525 / 0.519: straight.
+constexpr bool plane_mapped(int type, int kind, int prec, int cpq) {
+    return plane_always(type, kind, prec, cpq) && (type == TET ? kind == POISSON : prec == FP64 || kind == GENERIC);
+}
 
 // Fix-up kernels (flagged elements of the mixed and double-word forms, redone
 // with the Jacobian terms in double); they read the list written by the main kernel.

@@ -435,7 +435,8 @@ fe_status launch_set(fe_ctx *ctx, fe_elem_type type, const fe_elem_args *a, cons
     TmaMaps tm;
     memset(&tm, 0, sizeof tm);
     const bool soa_in = a->coords_layout == FE_LAYOUT_SOA, soa_out = o->layout == FE_LAYOUT_SOA;
-    bool planes = soa_in && soa_out && plane_always(type, a->kind, a->prec, cpq_of(a));
+    bool planes = soa_in && soa_out &&
+                  (mapped ? plane_mapped : plane_always)(type, a->kind, a->prec, cpq_of(a));
     if (!planes && sh.block <= 256) {
         const int ns = ns_of(type), nc = nc_of(type, a);
         const bool dbl = a->prec != FE_FP32_MIXED;

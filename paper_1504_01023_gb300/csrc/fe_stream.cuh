@@ -191,7 +191,7 @@ __global__ void __launch_bounds__(512) __maxnreg__(KIND == POISSON ? 64 : 128)
 template <int KIND, int QUAD, int CPQ, int INL, int OUTL> const void *f64_tet_kernel() {
     if constexpr (INL == AOS && OUTL == AOS && (CPQ == 0 || (CPQ == 1 && KIND == POISSON)))
         return reinterpret_cast<const void *>(&stream_kernel_f64t<KIND, QUAD, CPQ>);
-    else if constexpr (INL == SOA && out_soa(OUTL) && plane_always(TET, KIND, FP64, CPQ))
+    else if constexpr (INL == SOA && out_soa(OUTL) && plane_mapped(TET, KIND, FP64, CPQ))
         return nullptr;
     else
         return reinterpret_cast<const void *>(&elem_kernel_f64t<KIND, QUAD, CPQ, INL, OUTL>);
